@@ -140,15 +140,18 @@ rf_status check_volume_args(const rf_params* p, int64_t n_buckets, int64_t max_b
   return RF_OK;
 }
 
+// Partial-sum slots per word: the most chunks any registration level has (see
+// chunk_pixels in rf_track.cu: chunks of at least 128 pixels, at most
+// kRegChunks of them).
+size_t reg_slots(size_t npix) { return std::min<size_t>(kRegChunks, (npix + 127) / 128); }
+
 // Every device buffer of a volume, in one list: rf_create_volume allocates
 // them, rf_volume_footprint adds up their sizes.
 template <class Alloc>
 rf_status volume_buffers(rf_volume* vol, const rf_params* p, int64_t n_buckets, int64_t max_blocks, int max_width,
                          int max_height, Alloc&& A) {
   const size_t npix = (size_t)max_width * max_height;
-  // partial-sum slots per component: the chunks of the smallest registration
-  // chunk (128 pixels)
-  const size_t max_slots = (npix + 127) / 128;
+  const size_t max_slots = reg_slots(npix);
   const size_t ntiles = ((size_t)(max_width + kTile - 1) / kTile) * ((max_height + kTile - 1) / kTile);
   const size_t nslots = (size_t)n_buckets * kSlots;
   rf_status s;
@@ -157,11 +160,13 @@ rf_status volume_buffers(rf_volume* vol, const rf_params* p, int64_t n_buckets, 
       (s = A(&vol->d_coords, (size_t)max_blocks, "coords")) ||
       (s = A(&vol->d_nbr, 2 * (size_t)max_blocks, "neighbour tables")) || (s = A(&vol->d_nblocks, 1, "pool")) ||
       (s = A(&vol->d_status, 1, "status")) || (s = A(&vol->d_regtags, 3, "registration tags")) ||
-      (s = A(&vol->d_partials, 2 * 29 * max_slots, "partials")) || (s = A(&vol->d_seeds, npix, "seeds")) ||
+      (s = A(&vol->d_partials, 2 * kRegWords * max_slots, "partials")) || (s = A(&vol->d_seeds, npix, "seeds")) ||
       (s = A(&vol->d_md, npix, "mask work")) || (s = A(&vol->d_ff, (size_t)p->max_ff_sweeps + 2, "flood-fill words")) ||
       (s = A(&vol->d_integ, 1, "integ")) || (s = A(&vol->d_tilemax, ntiles, "tiles")) ||
       (s = A(&vol->d_dmask, npix, "masked depth")) ||
-      (s = A(&vol->d_cand, (size_t)p->max_candidates, "candidates")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
+      // (a registration keeps its pixel records in the candidate list's memory:
+      // the two never run at the same time on one volume)
+      (s = A(&vol->d_cand, std::max((size_t)p->max_candidates, npix), "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
       (s = A(&vol->d_rgb, npix * 3, "rgb staging")) || (s = A(&vol->d_mask, npix, "mask staging")) ||
       (s = A(&vol->d_T, 48, "poses")) || (s = A(&vol->d_info, 1, "info")) || (s = A(&vol->d_guard, 1, "guard count")) ||
       (s = A(&vol->d_pxcache, npix, "pixel block cache")))
@@ -674,7 +679,7 @@ rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_bl
     return s;
   }
   const size_t npix = (size_t)max_width * max_height;
-  vol->max_slots = (int)((npix + 127) / 128);
+  vol->max_slots = (int)reg_slots(npix);
   vol->reg_grid = register_max_grid(vol->device);
   if (vol->reg_grid > vol->sm_count) vol->reg_grid = vol->sm_count;
   if (vol->reg_grid < 1) {
@@ -710,7 +715,7 @@ rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_bl
   // registration tags start at 0 (base, counts) with every partial-sum word's tag 0
   if (!s) s = check_cuda(vol, cudaMemset(vol->d_regtags, 0, 3 * sizeof(unsigned)), "tag reset");
   if (!s)
-    s = check_cuda(vol, cudaMemset(vol->d_partials, 0, (size_t)2 * 29 * vol->max_slots * sizeof(unsigned long long)),
+    s = check_cuda(vol, cudaMemset(vol->d_partials, 0, (size_t)2 * kRegWords * vol->max_slots * sizeof(ulonglong2)),
                    "partials reset");
   if (!s) s = check_cuda(vol, cudaDeviceSynchronize(), "create sync");
   if (s) {
@@ -1040,7 +1045,7 @@ rf_status rf_set_registration_tag_base(rf_volume* vol, uint32_t base) {
                      (unsigned long long)span);
   rf_status s = check_cuda(vol, cudaDeviceSynchronize(), "tag base sync");
   if (!s)
-    s = check_cuda(vol, cudaMemset(vol->d_partials, 0, (size_t)2 * 29 * vol->max_slots * sizeof(unsigned long long)),
+    s = check_cuda(vol, cudaMemset(vol->d_partials, 0, (size_t)2 * kRegWords * vol->max_slots * sizeof(ulonglong2)),
                    "partials reset");
   const unsigned words[3] = {base, 0u, 0u};
   if (!s) s = check_cuda(vol, cudaMemcpy(vol->d_regtags, words, sizeof(words), cudaMemcpyHostToDevice), "tag base");

@@ -4,23 +4,25 @@
 // over three pixel sub-samplings (strides), coarse to fine.
 //
 // A whole registration (three levels, every LM iteration) is ONE cooperative
-// launch of k_register, one CTA of 512 threads per SM.  Per cost evaluation:
-//   1. every thread takes sampled pixels: Eq. 1 back-projection, rigid
-//      transform, hash lookup of the 8 lattice corners, trilinear SDF and
-//      intensity with analytic gradients, residuals and Jacobians
-//      J = dV/dp [I | -[p]x] (left perturbation);
+// launch of k_register, one CTA of 512 threads per SM.  At the start of a
+// level every thread writes the records of its sampled pixels (camera point
+// and intensity) into a per-volume buffer that only it reads again.  Per cost
+// evaluation:
+//   1. every thread takes its pixels' records: rigid transform, hash lookup of
+//      the 8 lattice corners, trilinear SDF and intensity with analytic
+//      gradients, residuals and Jacobians J = dV/dp [I | -[p]x] (left
+//      perturbation), the SDF and the colour term side by side in packed FP32;
 //   2. a warp-shuffle + shared-memory reduction of the 21 entries of J^T J,
 //      the 6 of J^T r, the cost and the valid count gives one FP32 partial
 //      per fixed chunk of pixels, written with the evaluation's tag;
 //   3. EVERY CTA reads all partials, each until it carries the tag (this is
 //      the only grid-wide wait, bounded), reduces them (FP32, the same fixed
 //      order) and runs the same LM step on its shared-memory copy of the LM
-//      state, on one warp: accept or reject the candidate (mean cost E/N must
-//      decrease), update lambda, solve the damped 6x6 system and compose the
-//      next candidate pose exp(delta) T (FP32 with exactly formed residuals
-//      and a pose carried as float pairs; see lm_step_warp).  Identical
-//      inputs and code give identical states in all CTAs, so no broadcast is
-//      needed.
+//      state: accept or reject the candidate (mean cost E/N must decrease),
+//      update lambda, solve the damped 6x6 system and compose the next
+//      candidate pose exp(delta) T (FP32 with exactly formed residuals and a
+//      pose carried as float pairs; see lm_candidate).  Identical inputs and
+//      code give identical states in all CTAs, so no broadcast is needed.
 // The LM state never leaves shared memory; a level ends early when the step
 // falls below the thresholds.  Results are deterministic: fixed chunks, fixed
 // pixel-to-thread mapping, fixed reduction order.
@@ -32,150 +34,218 @@
 namespace rf {
 namespace {
 
-__device__ __forceinline__ float lerpf(float a, float b, float t) { return a * (1.0f - t) + b * t; }
+// ---------------------------------------------------------------------------
+// Packed FP32: one instruction works on two floats, here the SDF term (low)
+// and the colour term (high) of a sample.  The registration issues about half
+// as many arithmetic instructions this way; it is bound by instruction issue
+// and latency, not by the FP32 pipes.
+// ---------------------------------------------------------------------------
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpk(f2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
+  f2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 
-// Trilinear SDF/intensity lookup with analytic gradients (per metre).
-// Corner n = dx + 2 dy + 4 dz.  Returns false unless all 8 corners exist and
-// were observed; *colour is true when all 8 also carry colour.
-// cached: the pixel's (key << 22 | pool) from an earlier sample, ~0 if none;
-// *fresh receives a new entry when the block had to be looked up.
+// Normal equations of one thread's samples: the 21 entries of J^T J, the 6 of
+// J^T r and the cost, each as (SDF sum, colour sum), and the valid count.
+struct Acc {
+  f2 v[28];
+  float n;
+};
+
+// The per-sample constants of a registration (uniform over the CTA).
+struct SampleConst {
+  float inv_voxel;
+  float sdf_scale;   // stored SDF -> metres
+  float gs_sdf;      // gradient of the stored SDF per voxel -> per metre
+  float col_scale;   // stored intensity -> sqrt(w_c) times intensity
+  float gs_col;      // its gradient
+};
+
+constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: adding it leaves an integer in the low mantissa bits
+constexpr float kBias = 8388608.0f;    // 2^23
+
+// One sample: the pixel's camera point (x, y, z) and offset `off` (minus
+// sqrt(w_c) times its intensity), looked up in the model at the pose `pose`
+// (rows of R | t) and added to the normal equations when its 8 corners exist
+// and were observed (corner n = dx + 2 dy + 4 dz); the colour term is added
+// when all 8 also carry colour.  cached: the pixel's (key << 22 | pool) from
+// an earlier sample, ~0 if none; returns the entry to keep when the block had
+// to be looked up, else ~0.
+//
+// A third of the cells straddle a block border, and in most warps some lane's
+// does.  All lanes therefore fetch their corners with the same eight loads
+// from (pool, index) pairs; only the neighbour table's two loads are
+// conditional.
 template <int ST>
-__device__ __forceinline__ bool model_sample(const DevVol& v, const DevParams& p, float px, float py, float pz,
-                                             float* V, float gV[3], float* I, float gI[3], bool* colour,
-                                             unsigned long long cached, unsigned long long* fresh) {
-  const float qx = px * p.inv_voxel, qy = py * p.inv_voxel, qz = pz * p.inv_voxel;
-  if (!(fabsf(qx) < 1.0e6f && fabsf(qy) < 1.0e6f && fabsf(qz) < 1.0e6f)) return false;
-  const float fkx = floorf(qx), fky = floorf(qy), fkz = floorf(qz);
-  const int kx = (int)fkx, ky = (int)fky, kz = (int)fkz;
-  const float fx = qx - fkx, fy = qy - fky, fz = qz - fkz;
-  const int lx = kx & 7, ly = ky & 7, lz = kz & 7;
+__device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const SampleConst& c, const float4* pose,
+                                                         float x, float y, float z, float off,
+                                                         unsigned long long cached, Acc& acc) {
+  const float4 r0 = pose[0], r1 = pose[1], r2 = pose[2];
+  const float px = fmaf(r0.z, z, fmaf(r0.y, y, r0.x * x)) + r0.w;
+  const float py = fmaf(r1.z, z, fmaf(r1.y, y, r1.x * x)) + r1.w;
+  const float pz = fmaf(r2.z, z, fmaf(r2.y, y, r2.x * x)) + r2.w;
+  const float qx = px * c.inv_voxel, qy = py * c.inv_voxel, qz = pz * c.inv_voxel;
+  // block coordinates within +-kMaxCoord (a NaN fails too); |q| < 2^22 then
+  // makes the rounding trick below an exact floor
+  constexpr float kLo = -8.0f * kMaxCoord, kHi = 8.0f * kMaxCoord + 8.0f;
+  if (!(qx >= kLo && qy >= kLo && qz >= kLo && qx < kHi && qy < kHi && qz < kHi)) return kEmpty;
+  const float tx = __fadd_rd(qx, kRound), ty = __fadd_rd(qy, kRound), tz = __fadd_rd(qz, kRound);
+  const int kx = __float_as_int(tx) - 0x4B400000, ky = __float_as_int(ty) - 0x4B400000,
+            kz = __float_as_int(tz) - 0x4B400000;
+  const float fx = qx - (tx - kRound), fy = qy - (ty - kRound), fz = qz - (tz - kRound);
   const int bx = kx >> 3, by = ky >> 3, bz = kz >> 3;
-  // FP32 storage: the uint2 words; FP16 storage: the 4-byte tracking words
-  using Word = typename std::conditional<ST == RF_STORAGE_FP32, uint2, unsigned>::type;
-  Word c[8];
-  if (!coord_ok(bx, by, bz)) return false;
-  const unsigned long long key = pack_key(bx, by, bz);
+  // the cached entry's upper 42 bits are the block key (bx, by, bz: 14 bits each)
+  const unsigned khi = ((unsigned)bx << 18) | (((unsigned)by & 0x3FFFu) << 4) | (((unsigned)bz >> 10) & 15u);
+  const unsigned klo = (unsigned)bz << 22;
+  const unsigned chi = (unsigned)(cached >> 32), clo = (unsigned)cached;
+  unsigned long long fresh = kEmpty;
   int pool;
-  if (cached != kEmpty && (cached >> 22) == key) {
-    pool = (int)(cached & 0x3FFFFFull);  // same block as last time: no hash probe
+  if (chi == khi && (clo ^ klo) < (1u << 22) && cached != kEmpty) {
+    pool = (int)(clo & 0x3FFFFFu);  // same block as last time: no hash probe
   } else {
     pool = hash_find(v, bx, by, bz);
-    if (pool < 0) return false;
-    *fresh = (key << 22) | (unsigned long long)pool;
+    if (pool < 0) return kEmpty;
+    fresh = ((unsigned long long)khi << 32) | klo | (unsigned)pool;
   }
-  const Word* words = reinterpret_cast<const Word*>(v.vox);
-  const size_t stride = ST == RF_STORAGE_FP32 ? kBV : 2 * kBV;  // words per block
-  if (lx < 7 && ly < 7 && lz < 7) {
-    const Word* base = words + (size_t)pool * stride + lx + 8 * ly + 64 * lz;
-    c[0] = __ldg(base);
-    c[1] = __ldg(base + 1);
-    c[2] = __ldg(base + 8);
-    c[3] = __ldg(base + 9);
-    c[4] = __ldg(base + 64);
-    c[5] = __ldg(base + 65);
-    c[6] = __ldg(base + 72);
-    c[7] = __ldg(base + 73);
-  } else {
-    // the cell straddles blocks: the neighbours' pools come from the table
+  const int lx = kx & 7, ly = ky & 7, lz = kz & 7;
+  int a0 = pool, a1 = pool, a2 = pool, a3 = pool;  // pools of the corners at dx = 0: (dy, dz) = 00, 10, 01, 11
+  int b0 = pool, b1 = pool, b2 = pool, b3 = pool;  // and at dx = 1
+  if (lx == 7 || ly == 7 || lz == 7) {
     const int4 n0 = __ldg(v.nbr + 2 * (size_t)pool), n1 = __ldg(v.nbr + 2 * (size_t)pool + 1);
     const bool ex = lx == 7, ey = ly == 7, ez = lz == 7;
-    int pn[8];
-    bool present = true;
+    const int m0 = ex ? n0.y : n0.x, m1 = ex ? n0.w : n0.z, m2 = ex ? n1.y : n1.x, m3 = ex ? n1.w : n1.z;
+    a1 = ey ? n0.z : n0.x;
+    a2 = ez ? n1.x : n0.x;
+    a3 = ez ? (ey ? n1.z : n1.x) : a1;
+    b0 = m0;
+    b1 = ey ? m1 : m0;
+    b2 = ez ? m2 : m0;
+    b3 = ez ? (ey ? m3 : m2) : b1;
+    if (min(min(min(a1, a2), min(a3, b0)), min(b1, min(b2, b3))) < 0) return fresh;
+  }
+  // FP32 storage: the uint2 words; FP16 storage: the 4-byte tracking words
+  using Word = typename std::conditional<ST == RF_STORAGE_FP32, uint2, unsigned>::type;
+  constexpr unsigned kStride = ST == RF_STORAGE_FP32 ? kBV : 2 * kBV;  // words per block
+  const Word* words = reinterpret_cast<const Word*>(v.vox);
+  const unsigned x1 = (unsigned)(lx + 1) & 7u, y0 = (unsigned)ly * 8u, y1 = ((unsigned)(ly + 1) & 7u) * 8u;
+  const unsigned z0 = (unsigned)lz * 64u, z1 = ((unsigned)(lz + 1) & 7u) * 64u;
+  Word w[8];  // (a 32-bit word index reaches every block: 2^22 blocks of 1,024 words)
+  w[0] = __ldg(words + ((unsigned)a0 * kStride + (lx + y0 + z0)));
+  w[1] = __ldg(words + ((unsigned)b0 * kStride + (x1 + y0 + z0)));
+  w[2] = __ldg(words + ((unsigned)a1 * kStride + (lx + y1 + z0)));
+  w[3] = __ldg(words + ((unsigned)b1 * kStride + (x1 + y1 + z0)));
+  w[4] = __ldg(words + ((unsigned)a2 * kStride + (lx + y0 + z1)));
+  w[5] = __ldg(words + ((unsigned)b2 * kStride + (x1 + y0 + z1)));
+  w[6] = __ldg(words + ((unsigned)a3 * kStride + (lx + y1 + z1)));
+  w[7] = __ldg(words + ((unsigned)b3 * kStride + (x1 + y1 + z1)));
+  // corner pairs (SDF, intensity), the intensity with 2^23 added (exact: it is
+  // a small integer), which cancels in the differences along x
+  f2 d[4], e[4];  // differences along x, and values at fx, of the four x edges
+  bool colour;
+  {
+    float I[8], F[8];
+    if constexpr (ST == RF_STORAGE_FP32) {
+      unsigned m = w[0].y;
 #pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      pn[n] = nbr_pick(n0, n1, (n & 1) && ex, ((n >> 1) & 1) && ey, ((n >> 2) & 1) && ez);
-      present = present && pn[n] >= 0;
+      for (int n = 0; n < 8; ++n) {
+        m = min(m, w[n].y);
+        F[n] = __uint_as_float(w[n].x);
+        I[n] = __uint_as_float(__dp2a_hi(722u, w[n].y, __dp2a_lo(2126u | (7152u << 16), w[n].y, 0x4B000000u)));
+      }
+      colour = m >= (1u << 24);  // the smallest colour weight (top byte) is not 0
+    } else {
+      unsigned m = 0u;
+#pragma unroll
+      for (int n = 0; n < 8; ++n) {
+        const unsigned i8 = (w[n] >> 16) & 255u;  // intensity x 254; 255 marks a corner without colour
+        m = max(m, i8);
+        F[n] = __half2float(__ushort_as_half((unsigned short)(w[n] & 0xFFFFu)));
+        I[n] = __uint_as_float(0x4B000000u | i8);
+      }
+      colour = m != 255u;
     }
-    if (!present) return false;
+    const f2 fx2 = pk(fx, fx);
 #pragma unroll
-    for (int n = 0; n < 8; ++n) {
-      const int ix = (lx + (n & 1)) & 7, iy = (ly + ((n >> 1) & 1)) & 7, iz = (lz + ((n >> 2) & 1)) & 7;
-      c[n] = __ldg(words + (size_t)pn[n] * stride + ix + 8 * iy + 64 * iz);
+    for (int n = 0; n < 4; ++n) {
+      d[n] = sub2(pk(F[2 * n + 1], I[2 * n + 1]), pk(F[2 * n], I[2 * n]));
+      e[n] = fma2(fx2, d[n], pk(F[2 * n], I[2 * n] - kBias));
     }
   }
-  float F[8];
-  if constexpr (ST == RF_STORAGE_FP32) {
-#pragma unroll
-    for (int n = 0; n < 8; ++n) F[n] = __uint_as_float(c[n].x);
-  } else {
-#pragma unroll
-    for (int n = 0; n < 8; ++n) F[n] = __half2float(__ushort_as_half((unsigned short)(c[n] & 0xFFFFu)));
-  }
-  // FP16 storage holds F / tau: values and gradients are scaled by tau once
-  const float sdf_scale = ST == RF_STORAGE_FP32 ? 1.0f : p.tau;
-  const float c00 = lerpf(F[0], F[1], fx), c10 = lerpf(F[2], F[3], fx);
-  const float c01 = lerpf(F[4], F[5], fx), c11 = lerpf(F[6], F[7], fx);
-  const float c0 = lerpf(c00, c10, fy), c1 = lerpf(c01, c11, fy);
-  *V = lerpf(c0, c1, fz) * sdf_scale;
-  // a never-observed corner stores NaN; every corner enters V with its
-  // weight (0 * NaN = NaN), so one test covers all eight
-  if (*V != *V) return false;
-  const float gs_v = p.inv_voxel * sdf_scale;
-  gV[0] = lerpf(lerpf(F[1] - F[0], F[3] - F[2], fy), lerpf(F[5] - F[4], F[7] - F[6], fy), fz) * gs_v;
-  gV[1] = lerpf(lerpf(F[2] - F[0], F[3] - F[1], fx), lerpf(F[6] - F[4], F[7] - F[5], fx), fz) * gs_v;
-  gV[2] = (c1 - c0) * gs_v;
-  float In[8];
-  float iscale;
-  if constexpr (ST == RF_STORAGE_FP32) {
-    // colour weights in the top bytes: their minimum over the corners
-    const unsigned wmin = __vminu4(__vminu4(__vminu4(c[0].y, c[1].y), __vminu4(c[2].y, c[3].y)),
-                                   __vminu4(__vminu4(c[4].y, c[5].y), __vminu4(c[6].y, c[7].y)));
-    *colour = (wmin >> 24) != 0u;
-    if (!*colour) return true;
-#pragma unroll
-    for (int n = 0; n < 8; ++n) In[n] = rgb_intensity_raw(c[n].y);  // intensities x 255e4
-    iscale = kIntensityScale;
-  } else {
-    // I8 = 255 marks a corner without colour: the byte maximum over the corners
-    const unsigned imax = __vmaxu4(__vmaxu4(__vmaxu4(c[0], c[1]), __vmaxu4(c[2], c[3])),
-                                   __vmaxu4(__vmaxu4(c[4], c[5]), __vmaxu4(c[6], c[7])));
-    *colour = ((imax >> 16) & 255u) != 255u;
-    if (!*colour) return true;
-#pragma unroll
-    for (int n = 0; n < 8; ++n) In[n] = u2f_exact((c[n] >> 16) & 255u);  // intensities x 254
-    iscale = kI8Scale;
-  }
-  const float d00 = lerpf(In[0], In[1], fx), d10 = lerpf(In[2], In[3], fx);
-  const float d01 = lerpf(In[4], In[5], fx), d11 = lerpf(In[6], In[7], fx);
-  const float d0 = lerpf(d00, d10, fy), d1 = lerpf(d01, d11, fy);
-  const float gs = iscale * p.inv_voxel;
-  *I = lerpf(d0, d1, fz) * iscale;
-  gI[0] = lerpf(lerpf(In[1] - In[0], In[3] - In[2], fy), lerpf(In[5] - In[4], In[7] - In[6], fy), fz) * gs;
-  gI[1] = lerpf(lerpf(In[2] - In[0], In[3] - In[1], fx), lerpf(In[6] - In[4], In[7] - In[5], fx), fz) * gs;
-  gI[2] = (d1 - d0) * gs;
-  return true;
-}
-
-__device__ __forceinline__ void add_jtj(float* acc, const float J[6], float r, float w) {
+  const f2 fy2 = pk(fy, fy), fz2 = pk(fz, fz);
+  const f2 gy0 = sub2(e[1], e[0]), gy1 = sub2(e[3], e[2]);
+  const f2 c0 = fma2(fy2, gy0, e[0]), c1 = fma2(fy2, gy1, e[2]);
+  f2 gz = sub2(c1, c0);
+  const f2 val = fma2(fz2, gz, c0);
+  float V, I;
+  unpk(val, V, I);
+  // a never-observed corner stores NaN; every corner enters V, so one test
+  // covers all eight
+  if (V != V) return fresh;
+  f2 gy = fma2(fz2, sub2(gy1, gy0), gy0);
+  const f2 d0 = fma2(fy2, sub2(d[1], d[0]), d[0]), d1 = fma2(fy2, sub2(d[3], d[2]), d[2]);
+  f2 gx = fma2(fz2, sub2(d1, d0), d0);
+  const f2 gs = pk(c.gs_sdf, colour ? c.gs_col : 0.0f);
+  gx = mul2(gx, gs);
+  gy = mul2(gy, gs);
+  gz = mul2(gz, gs);
+  const f2 r = fma2(val, pk(c.sdf_scale, colour ? c.col_scale : 0.0f), pk(0.0f, colour ? off : 0.0f));
+  f2 J[6];
+  J[0] = gx;
+  J[1] = gy;
+  J[2] = gz;
+  J[3] = fma2(pk(py, py), gz, mul2(pk(-pz, -pz), gy));
+  J[4] = fma2(pk(pz, pz), gx, mul2(pk(-px, -px), gz));
+  J[5] = fma2(pk(px, px), gy, mul2(pk(-py, -py), gx));
   int n = 0;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const float wi = w * J[i];
+  for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int j = i; j < 6; ++j) acc[n++] += wi * J[j];
-  }
+    for (int j = i; j < 6; ++j) {
+      acc.v[n] = fma2(J[i], J[j], acc.v[n]);
+      ++n;
+    }
 #pragma unroll
-  for (int i = 0; i < 6; ++i) acc[21 + i] += w * J[i] * r;
-  acc[27] += w * r * r;
+  for (int i = 0; i < 6; ++i) acc.v[21 + i] = fma2(J[i], r, acc.v[21 + i]);
+  acc.v[27] = fma2(r, r, acc.v[27]);
+  acc.n += 1.0f;
+  return fresh;
 }
 
-
 // LM state of one registration, one copy in the shared memory of every CTA.
+// Poses are kept as pairs of floats per entry (hi + lo, about 48 bits; hi is
+// the float pose an evaluation uses), rows (R | t) of four.
 struct LMShared {
-  float Ef;       // FP32 cost sum E of the accepted pose
-  long long N, fin_N;
+  float sums[2][32];    // FP32 sums of an evaluation: 21 of J^T J, 6 of J^T r, cost, valid count; one slot holds the
+                        // accepted pose's, the other the evaluation just reduced
+  float4 pose[4][3];    // hi parts: the accepted pose, the candidate, and the two possible next candidates
+  float4 plo[4][3];     // lo parts
+  int stop[2];          // next candidate after an acceptance / a rejection: 1 when there is none (level converged)
+  int accept;
+  float E;              // cost and valid count of the accepted pose
+  unsigned N;
   float fin_E;
-  int lam_k;            // damping lambda0 * 10^lam_k
-  float Hf[21], gf[6];  // normal equations of the accepted pose (FP32 sums)
-  float redf[29];       // FP32 sums of the partials of the evaluation just reduced
-  // the accepted pose T and the candidate Tc (R row-major, then t), each
-  // entry an unevaluated sum hi + lo of two floats (about 48 bits): hi is the
-  // float pose an evaluation uses, hi + lo the pose itself
-  float Rf[12], Rlf[12];
-  float Rcf[12], Rclf[12];
-  double T0[12];  // the initial pose, returned unchanged when no candidate is accepted
-  int moved;      // some candidate was accepted
-  int done;
+  unsigned fin_N;
+  double T0[12];        // the initial pose, returned unchanged when no candidate is accepted
   rf_track_info info;
 };
 
@@ -188,31 +258,27 @@ __host__ __device__ constexpr int up6(int i, int j) { return i * 6 - i * (i - 1)
 // upper triangle (row-major) on entry and L^T (L's column j stored as row j of
 // the upper triangle) on exit; inv[j] = 1 / L[j][j] from the hardware
 // reciprocal square root (the factor only preconditions the refined solve).
-// False unless every pivot is positive and finite.  Fully unrolled.
+// False unless every pivot is positive and finite.  Right-looking (a pivot's
+// updates of the trailing rows are independent of one another, so the chain
+// from pivot to pivot is one reciprocal square root and three operations);
+// constant bounds with guards unroll fully and keep A in registers.
 __device__ __forceinline__ bool chol6(float A[21], float inv[6]) {
-  // every loop has constant bounds (with guards) so that it unrolls fully and
-  // A stays in registers
   bool ok = true;
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    float s = A[up6(j, j)];
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (k < j) s = fmaf(-A[up6(k, j)], A[up6(k, j)], s);
+    const float s = A[up6(j, j)];
     ok = ok && (s > 0.0f) && (s < 3.0e38f);
     const float r = rsqrtf(fmaxf(s, 1.0e-30f));
     A[up6(j, j)] = s * r;
     inv[j] = r;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      if (i > j) {
-        float t = A[up6(j, i)];
+    for (int i = 0; i < 6; ++i)
+      if (i > j) A[up6(j, i)] *= r;
 #pragma unroll
-        for (int k = 0; k < 6; ++k)
-          if (k < j) t = fmaf(-A[up6(k, i)], A[up6(k, j)], t);
-        A[up6(j, i)] = t * r;
-      }
-    }
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (i > j && k >= i) A[up6(i, k)] = fmaf(-A[up6(j, i)], A[up6(j, k)], A[up6(i, k)]);
   }
   return ok;
 }
@@ -264,76 +330,37 @@ __device__ __forceinline__ bool prod_less(float a, unsigned na, float b, unsigne
   return xa >= xb ? (P << (xa - xb)) < Q : P < (Q << (xb - xa));
 }
 
-// One LM step, executed by the 32 lanes of one warp.  On GB300 a dependent
-// FP64 instruction costs hundreds of cycles (measured with clock64 stamps in
-// this loop: about 300-400 per dependent FP64 operation), and the step lies
-// on the registration's serial critical path; so the step works in FP32 and
-// reaches FP64-class accuracy where it matters without FP64 latency:
-//   mode 0: first evaluation of a level, at T (always taken);
-//   mode 1: evaluation of the candidate Tc, accepted when the mean cost
-//           decreases (En/Nn < E/N, compared exactly as En N < E Nn on the
-//           integer mantissas);
-//   damping lambda = lambda0 10^k, k counting rejections minus acceptances;
-//   solve of (H + lambda diag H) d = -g: FP32 Cholesky, then one step of
-//   iterative refinement whose residual -g - A d is formed exactly (FP32
-//   error-free transformations: the products of FP32 numbers and their sum
-//   carried to about 2^-46), which gives the solution to the accuracy of an
-//   FP64 solve for the systems met here (condition numbers ~10^2);
+// The next candidate pose of the LM iteration, executed by the 32 lanes of one
+// warp: solves (H + lambda diag H) d = -g for the sums of an evaluation at the
+// pose (hi, lo) and writes exp(d) T to (out, out_lo).  Returns true when there
+// is no next candidate: the step is below the thresholds or the solve failed.
+//
+// On GB300 a dependent FP64 instruction costs hundreds of cycles (measured
+// with clock64 stamps in this loop: about 300-400 per dependent FP64
+// operation), and the step lies on the registration's serial critical path;
+// so the step works in FP32 and reaches FP64-class accuracy where it matters
+// without FP64 latency:
+//   solve: FP32 Cholesky, then one step of iterative refinement whose residual
+//   -g - A d is formed exactly (FP32 error-free transformations: the products
+//   of FP32 numbers and their sum carried to about 2^-46), which gives the
+//   solution to the accuracy of an FP64 solve for the systems met here
+//   (condition numbers ~10^2);
 //   exp(d) - I = [A K + B K^2 | rho + B K rho + C K^2 rho] in FP32 (its
 //   entries are of the order of the step, so FP32 is relative to the step);
-//   the candidate pose Tc = T + (exp(d) - I) T: the increment in FP32, added
+//   the candidate pose T + (exp(d) - I) T: the increment in FP32, added
 //   to the pose carried as float pairs with an error-free sum (lanes 0-11 in
 //   parallel); the pair's high float is what the next evaluation uses.
-__device__ void lm_step_warp(LMShared& S, int mode, int level, bool last, const LMConst& c, int lane) {
-  const float Enf = S.redf[27];
-  const long long Nn = (long long)(S.redf[28] + 0.5f);
-  int accept;
-  bool done = false;
-  int k = S.lam_k;
-  if (mode == 0) {
-    accept = 1;
-    k = 0;
-    done = Nn < c.min_valid;
-  } else if (Nn >= c.min_valid && prod_less(Enf, (unsigned)S.N, S.Ef, (unsigned)Nn)) {  // N < 2^24
-    accept = 2;
-    k = max(k - 1, -kLambdaPow);
-  } else {
-    accept = 0;
-    k = min(k + 1, kLambdaPow);
-  }
-  __syncwarp();  // every lane has read the state before lane 0 updates it
-  if (lane == 0) {
-    S.info.evals++;
-    S.info.level_evals[level]++;
-    S.lam_k = k;
-    if (accept) {
-      S.Ef = Enf;
-      S.N = Nn;
-      S.fin_E = Enf;
-      S.fin_N = Nn;
-    }
-    if (accept == 2) S.moved = 1;
-    if (mode == 0) S.done = done ? 1 : 0;  // every level starts undone unless it has too few pixels
-  }
-  if (accept) {
-    if (lane < 21) S.Hf[lane] = S.redf[lane];
-    else if (lane < 27) S.gf[lane - 21] = S.redf[lane];
-    if (accept == 2 && lane < 12) {
-      S.Rf[lane] = S.Rcf[lane];
-      S.Rlf[lane] = S.Rclf[lane];
-    }
-  }
-  __syncwarp();
-  if (done || last) return;  // (a candidate is only evaluated while the level is not done)
-  const float lam = c.lambda_pow[k + kLambdaPow];
-  // FP32 Cholesky of the damped matrix and first solution (every lane)
+// Not inlined: two warps call it (see register_body), and the instruction
+// cache holds one copy.
+__device__ __noinline__ bool lm_candidate(const float* sums, const float* hi, const float* lo, float lam, float eps_t2,
+                                          float eps_r2, float* out, float* out_lo, int lane) {
   float A[21], inv[6], d[6], r[6];
 #pragma unroll
-  for (int q = 0; q < 21; ++q) A[q] = S.Hf[q];
+  for (int q = 0; q < 21; ++q) A[q] = sums[q];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     A[up6(i, i)] = fmaf(A[up6(i, i)], lam, A[up6(i, i)]);
-    d[i] = -S.gf[i];
+    d[i] = -sums[21 + i];
   }
   const bool ok = chol6(A, inv);
   chol6_solve(A, inv, d);
@@ -341,10 +368,10 @@ __device__ void lm_step_warp(LMShared& S, int mode, int level, bool last, const 
   // lane i, then gathered on every lane
   {
     const int i = lane < 6 ? lane : 0;
-    float sh = -S.gf[i], sl = 0.0f;
+    float sh = -sums[21 + i], sl = 0.0f;
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const float h = S.Hf[i <= j ? up6(i, j) : up6(j, i)];
+      const float h = sums[i <= j ? up6(i, j) : up6(j, i)];
       float p, pe, e;
       two_prod(h, d[j], p, pe);
       two_sum(sh, -p, sh, e);
@@ -367,14 +394,7 @@ __device__ void lm_step_warp(LMShared& S, int mode, int level, bool last, const 
   const float nr2 = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
   const float p0 = d[3], p1 = d[4], p2 = d[5];
   const float t2 = fmaf(p0, p0, fmaf(p1, p1, p2 * p2));
-  if (!ok || !(nr2 < 3.0e38f) || !(t2 < 3.0e38f) || (nr2 < c.eps_t2f && t2 < c.eps_r2f)) {
-    if (lane == 0) {
-      S.info.converged[level] = 1;
-      S.done = 1;
-    }
-    __syncwarp();
-    return;
-  }
+  if (!ok || !(nr2 < 3.0e38f) || !(t2 < 3.0e38f) || (nr2 < eps_t2 && t2 < eps_r2)) return true;
   // exponential map minus identity: A, B, C of theta^2
   float cA, cB, cC;
   if (t2 < 0.01f) {  // Taylor series in theta^2, enough terms for FP32 below theta = 0.1
@@ -403,8 +423,7 @@ __device__ void lm_step_warp(LMShared& S, int mode, int level, bool last, const 
     const float e0 = fmaf(cA, k0, cB * fmaf(pi, p0, i == 0 ? -t2 : 0.0f));
     const float e1 = fmaf(cA, k1, cB * fmaf(pi, p1, i == 1 ? -t2 : 0.0f));
     const float e2 = fmaf(cA, k2, cB * fmaf(pi, p2, i == 2 ? -t2 : 0.0f));
-    const float c0 = S.Rf[j < 3 ? j : 9], c1 = S.Rf[j < 3 ? 3 + j : 10], c2 = S.Rf[j < 3 ? 6 + j : 11];
-    float inc = fmaf(e0, c0, fmaf(e1, c1, e2 * c2));
+    float inc = fmaf(e0, hi[j], fmaf(e1, hi[4 + j], e2 * hi[8 + j]));
     if (j == 3) {  // + (rho + B K rho + C K^2 rho)_i
       const float kr = fmaf(k0, d[0], fmaf(k1, d[1], k2 * d[2]));  // (K rho)_i
       const float kr0 = p1 * d[2] - p2 * d[1], kr1 = p2 * d[0] - p0 * d[2], kr2 = p0 * d[1] - p1 * d[0];
@@ -412,66 +431,70 @@ __device__ void lm_step_warp(LMShared& S, int mode, int level, bool last, const 
       const float rho_i = i == 0 ? d[0] : (i == 1 ? d[1] : d[2]);
       inc += fmaf(cC, kk, fmaf(cB, kr, rho_i));
     }
-    const int fi = j < 3 ? i * 3 + j : 9 + i;
-    float hi, lo;
-    two_sum(S.Rf[fi], inc, hi, lo);
-    lo += S.Rlf[fi];
-    const float h2 = hi + lo;  // renormalised: h2 is the nearest float of the pair's sum
-    S.Rcf[fi] = h2;
-    S.Rclf[fi] = lo - (h2 - hi);
+    float sum, err;
+    two_sum(hi[lane], inc, sum, err);
+    err += lo[lane];
+    const float h2 = sum + err;  // renormalised: h2 is the nearest float of the pair's sum
+    out[lane] = h2;
+    out_lo[lane] = err - (h2 - sum);
   }
-  __syncwarp();
+  return false;
 }
 
 constexpr int kRegThreads = 512;
 constexpr int kRegWarps = kRegThreads / 32;
 
-// Pixels per partial sum: a fixed chunk of the sampled pixels of a level
-// (128 below 2^16 pixels, 512 below 2^18, else 2048), so the partials, and
-// thus the result, do not depend on how many CTAs run the registration.
+// Pixels per partial sum: a fixed chunk of the sampled pixels of a level, a
+// function of their number only, so the partials, and thus the result, do not
+// depend on how many CTAs run the registration.  At most kRegChunks chunks
+// (one per CTA of a registration that has the GPU to itself, 98.7 % of the
+// SMs), of at least 128 pixels and a whole number of warps.
 __device__ __forceinline__ int chunk_pixels(int npix) {
-  return npix >= (1 << 18) ? 4 * kRegThreads : (npix >= (1 << 16) ? kRegThreads : kRegThreads / 4);
+  const int c = (npix + kRegChunks - 1) / kRegChunks;
+  return max(128, (c + 127) & ~127);
 }
-constexpr int kMaxPerThread = 4;  // pixels of one chunk per thread (chunk_pixels / kRegThreads at most)
-constexpr int kReduceBatch = 8;   // partials per lane and component loaded at once in the reduction
 
-// The pixels of chunk ch that thread tin of its slot samples (at most
-// kMaxPerThread, kRegThreads apart): raw depth (0 where masked), (u, v) and
-// packed RGB, and the pixel's cached block entry.  All loads are issued
-// before any is used, so their latencies overlap.
-struct PixelRegs {
-  unsigned raw[kMaxPerThread], uv[kMaxPerThread], rgb[kMaxPerThread];
-  unsigned long long cache[kMaxPerThread];
+// Pixel index in the frame of sample i of a level (row = i / Ws by a
+// reciprocal multiply, off by at most one for i < 2^32, then corrected).
+struct LevelMap {
+  int Ws, stride, W;
+  unsigned long long magic;
+  __device__ __forceinline__ void locate(int i, int& u, int& v) const {
+    int row = (int)(((unsigned long long)i * magic) >> 32);
+    if (row * Ws > i) --row;
+    else if ((row + 1) * Ws <= i) ++row;
+    u = (i - row * Ws) * stride;
+    v = row * stride;
+  }
+  __device__ __forceinline__ int pixel(int i) const {
+    if (stride == 1) return i;
+    int u, v;
+    locate(i, u, v);
+    return v * W + u;
+  }
 };
 
-__device__ __forceinline__ void load_pixels(const RegDesc& d, PixelRegs& P, int ch, int chunk, int npix, int nchunks,
-                                            int Ws, unsigned long long magic, int stride, int tin) {
+// Record of sample i of a level, written once per level by the thread that
+// samples it: camera point of Eq. 1 and minus sqrt(w_c) times the intensity;
+// z = 0 where the pixel is not sampled (invalid depth or masked).
+__device__ __forceinline__ void write_record(const RegDesc& d, const LevelMap& m, float col_off, int i) {
   const DevFrame& f = d.f;
-  const int end = ch < nchunks ? min(npix, (ch + 1) * chunk) : 0;
-#pragma unroll
-  for (int j = 0; j < kMaxPerThread; ++j) {
-    const int i = ch * chunk + tin + j * kRegThreads;
-    P.raw[j] = 0u;
-    P.uv[j] = 0u;
-    P.rgb[j] = 0u;
-    P.cache[j] = kEmpty;
-    if (i < end) {
-      // row = i / Ws by a reciprocal multiply (off by at most one for
-      // i < 2^32), then one integer correction step
-      int row = (int)(((unsigned long long)i * magic) >> 32);
-      if (row * Ws > i) --row;
-      else if ((row + 1) * Ws <= i) ++row;
-      const int u = (i - row * Ws) * stride, vv = row * stride;
-      const int idx = vv * f.W + u;
-      unsigned raw = __ldg(f.depth + idx);
-      if (d.mask && __ldg(d.mask + idx)) raw = 0u;  // masked: not sampled
-      const uint8_t* cp = f.rgb + 3 * (size_t)idx;
-      P.raw[j] = raw;
-      P.uv[j] = (unsigned)u | ((unsigned)vv << 16);
-      if (raw != 0u && d.pxcache) P.cache[j] = __ldcg(d.pxcache + idx);
-      P.rgb[j] = (unsigned)__ldg(cp) | ((unsigned)__ldg(cp + 1) << 8) | ((unsigned)__ldg(cp + 2) << 16);
-    }
+  int u, v;
+  m.locate(i, u, v);
+  const int idx = v * m.W + u;
+  unsigned raw = __ldg(f.depth + idx);
+  if (d.mask && __ldg(d.mask + idx)) raw = 0u;
+  const uint8_t* cp = f.rgb + 3 * (size_t)idx;
+  const unsigned rgb = (unsigned)__ldg(cp) | ((unsigned)__ldg(cp + 1) << 8) | ((unsigned)__ldg(cp + 2) << 16);
+  float4 r = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (pixel_valid(d.p, raw)) {
+    const float D = u2f_exact(raw) * d.p.inv_depth_scale;
+    r.x = (u2f_exact((unsigned)u) - f.cx) * f.ifx * D;
+    r.y = (u2f_exact((unsigned)v) - f.cy) * f.ify * D;
+    r.z = D;
+    r.w = rgb_intensity_raw(rgb) * col_off;
   }
+  d.rec[i] = r;
 }
 
 // Every CTA of a registration group calls this once, after its last read of
@@ -481,7 +504,7 @@ __device__ __forceinline__ void load_pixels(const RegDesc& d, PixelRegs& P, int 
 // the tags would reach kTagLimit it first clears the whole partial buffer,
 // whose tags then all read 0, and restarts the base at 0.  Either way every
 // tag left in the buffer is below the next registration's tags.
-__device__ __forceinline__ void leave_registration(const RegDesc& d, int lb, int G, unsigned tag0) {
+__device__ __forceinline__ void leave_registration(const RegDesc& d, int G, unsigned tag0) {
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(d.tags + 1, 1u) == (unsigned)G - 1u;
@@ -490,8 +513,8 @@ __device__ __forceinline__ void leave_registration(const RegDesc& d, int lb, int
   const unsigned span = (unsigned)(d.c.iters[0] + d.c.iters[1] + d.c.iters[2] + 3);
   unsigned next = tag0 + span;
   if (next >= kTagLimit - span) {
-    const size_t n = (size_t)2 * 29 * d.max_slots;
-    for (size_t i = threadIdx.x; i < n; i += kRegThreads) d.partials[i] = 0ull;
+    const int n = 2 * kRegWords * d.max_slots;
+    for (int i = threadIdx.x; i < n; i += kRegThreads) d.partials[i] = make_ulonglong2(0ull, 0ull);
     next = 0u;
   }
   if (threadIdx.x == 0) {
@@ -512,153 +535,186 @@ __device__ __forceinline__ void leave_registration(const RegDesc& d, int lb, int
 // so the tags carry the ordering).  The count also makes double buffering by
 // evaluation parity safe: a CTA writes evaluation e + 2 only after all G CTAs
 // arrived at e + 1, each after it had read all of evaluation e.
+//
+// The LM step is split over two warps so that little of it follows the
+// reduction: while the CTA waits for the others, warp 1 computes the next
+// candidate of a rejection (it needs the accepted pose's sums only); after
+// the reduction warp 0 computes the next candidate of an acceptance while
+// warp 1 decides which of the two applies.
 template <int ST>
 __device__ void register_body(const RegDesc& d, int lb, int G) {
   __shared__ LMShared S;
-  __shared__ float red[2][kRegWarps][29];  // per-warp sums of a chunk, double-buffered by step parity
+  __shared__ float red[2][kRegWarps][32];  // per-warp sums of a chunk, double-buffered by step parity
   __shared__ int s_arrived;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const DevFrame& f = d.f;
-  const DevParams& p = d.p;
 
   if (threadIdx.x == 0) {
-    S.done = 0;
-    S.Ef = 0.0f;
-    S.N = 0;
     S.fin_E = 0.0f;
-    S.fin_N = 0;
-    S.lam_k = 0;
-    S.moved = 0;
+    S.fin_N = 0u;
     rf_track_info z = {};
     S.info = z;
   }
-  __syncthreads();
   if (threadIdx.x < 12) {  // the initial pose as float pairs (FP64 once per registration)
-    const int i = threadIdx.x < 9 ? threadIdx.x / 3 : threadIdx.x - 9;
-    const int j = threadIdx.x < 9 ? threadIdx.x % 3 : 3;
-    const double t = d.T_init[i * 4 + j];
+    const double t = d.T_init[threadIdx.x];
     S.T0[threadIdx.x] = t;
     const float hi = (float)t;
-    S.Rf[threadIdx.x] = hi;
-    S.Rlf[threadIdx.x] = (float)(t - (double)hi);
-    S.Rcf[threadIdx.x] = hi;
-    S.Rclf[threadIdx.x] = S.Rlf[threadIdx.x];
+    reinterpret_cast<float*>(S.pose[0])[threadIdx.x] = hi;
+    reinterpret_cast<float*>(S.plo[0])[threadIdx.x] = (float)(t - (double)hi);
   }
+  SampleConst c;
+  {
+    const float swc = sqrtf(d.p.w_c);
+    c.inv_voxel = d.p.inv_voxel;
+    c.sdf_scale = ST == RF_STORAGE_FP32 ? 1.0f : d.p.tau;  // FP16 storage holds F / tau
+    c.gs_sdf = d.p.inv_voxel * c.sdf_scale;
+    c.col_scale = (ST == RF_STORAGE_FP32 ? kIntensityScale : kI8Scale) * swc;
+    c.gs_col = c.col_scale * d.p.inv_voxel;
+  }
+  const float col_off = -kIntensityScale * sqrtf(d.p.w_c);
   __syncthreads();
   const unsigned tag0 = ld_relaxed_gpu(d.tags);  // written by the previous registration's last CTA
   int eval = 0;
-  bool failed = false;
-  PixelRegs P;
+  bool failed = false, moved = false;
+  int iT = 0, iC = 1, iA = 2, iR = 3;  // pose slots: accepted, candidate, next after acceptance, next after rejection
+  int cur = 0;                         // slot of S.sums that holds the accepted pose's
   for (int l = 0; l < 3 && !failed; ++l) {
-    const int stride = d.c.strides[l];
-    const int Ws = (f.W + stride - 1) / stride, Hs = (f.H + stride - 1) / stride;
-    const int npix = Ws * Hs;
+    LevelMap m;
+    m.stride = d.c.strides[l];
+    m.W = f.W;
+    m.Ws = (f.W + m.stride - 1) / m.stride;
+    m.magic = (0x100000000ull + m.Ws - 1) / m.Ws;
+    const int npix = m.Ws * ((f.H + m.stride - 1) / m.stride);
     const int chunk = chunk_pixels(npix);
     const int nchunks = (npix + chunk - 1) / chunk;
-    const unsigned long long magic = (0x100000000ull + Ws - 1) / Ws;
     const int iters = d.c.iters[l];
-    bool pre = false;  // P already holds the pixels of the next step to run
-    for (int it = 0; it <= iters; ++it) {
-      const int mode = it == 0 ? 0 : 1;
-      if (mode == 1 && S.done) break;  // identical decision in every CTA of the group
-      const float* Tf = mode == 0 ? S.Rf : S.Rcf;
-      const float R0 = Tf[0], R1 = Tf[1], R2 = Tf[2], R3 = Tf[3], R4 = Tf[4], R5 = Tf[5], R6 = Tf[6], R7 = Tf[7],
-                  R8 = Tf[8], t0 = Tf[9], t1 = Tf[10], t2 = Tf[11];
-      unsigned long long* part = d.partials + (size_t)(eval & 1) * 29 * d.max_slots;
+    // chunks narrower than the CTA run side by side, one per warp group
+    // (slot): chunk lb + G (slot + slots step) at each step
+    const int width = min(chunk, kRegThreads);  // threads per chunk
+    const int slots = kRegThreads / width;
+    const int slot = threadIdx.x / width, tin = threadIdx.x - slot * width;
+    const int per_step = G * slots;
+    // this thread's samples of a chunk: first, first + width, ... below end
+    auto bounds = [&](int ch, int& end) {
+      end = slot < slots && ch < nchunks ? min(npix, (ch + 1) * chunk) : 0;
+      return ch * chunk + tin;
+    };
+    for (int ch = lb + G * slot; ch < nchunks && slot < slots; ch += per_step) {
+      int end;
+      for (int i = bounds(ch, end); i < end; i += width) write_record(d, m, col_off, i);
+    }
+    bool done = false;
+    int k = 0;  // damping lambda0 10^k: rejections minus acceptances
+    // the first sample's record of the next evaluation, loaded ahead of it
+    float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    unsigned long long cached = kEmpty;
+    {
+      int end;
+      const int i = bounds(lb + G * slot, end);
+      if (i < end) {
+        rec = d.rec[i];
+        cached = d.pxcache[m.pixel(i)];
+      }
+    }
+    for (int it = 0; it <= iters && !done; ++it) {
+      const bool first = it == 0, last = it == iters;
+      const float4* pose = S.pose[first ? iT : iC];
+      ulonglong2* part = d.partials + (size_t)(eval & 1) * kRegWords * d.max_slots;
       const unsigned tag = tag0 + (unsigned)eval + 1u;
-      // chunks narrower than the CTA run side by side, one per warp group
-      // (slot): chunk lb + G (slot + slots it) at step it
-      const int width = min(chunk, kRegThreads);  // threads per chunk
-      const int slots = kRegThreads / width;
-      const int slot = threadIdx.x / width, tin = threadIdx.x % width;
-      for (int step = 0; lb + G * slots * step < nchunks; ++step) {
-        const int ch = lb + G * (slot + slots * step);
-        float acc[29];
+      for (int step = 0; lb + per_step * step < nchunks; ++step) {
+        const int ch = lb + G * slot + per_step * step;
+        Acc acc;
 #pragma unroll
-        for (int i = 0; i < 29; ++i) acc[i] = 0.0f;
-        if (!pre) load_pixels(d, P, ch, chunk, npix, nchunks, Ws, magic, stride, tin);
+        for (int i = 0; i < 28; ++i) acc.v[i] = 0ull;
+        acc.n = 0.0f;
+        int end;
+        int i = bounds(ch, end);
+        const bool any = __any_sync(0xffffffffu, i < end);
 #pragma unroll 1
-        for (int j = 0; j < kMaxPerThread; ++j) {
-          // the next pixel's values rotate into slot 0 (registers, no local memory)
-          const unsigned raw = P.raw[0], uvj = P.uv[0], rgbj = P.rgb[0];
-          const unsigned long long cj = P.cache[0];
-#pragma unroll
-          for (int r = 0; r + 1 < kMaxPerThread; ++r) {
-            P.raw[r] = P.raw[r + 1];
-            P.uv[r] = P.uv[r + 1];
-            P.rgb[r] = P.rgb[r + 1];
-            P.cache[r] = P.cache[r + 1];
+        while (i < end) {
+          const float4 r = rec;
+          const unsigned long long cj = cached;
+          const int here = i;
+          i += width;
+          if (i < end) {  // the next sample's record
+            rec = d.rec[i];
+            cached = d.pxcache[m.pixel(i)];
           }
-          if (!pixel_valid(p, raw)) continue;
-          const int u = (int)(uvj & 0xFFFFu), vv = (int)(uvj >> 16);
-          const float D = u2f_exact(raw) * p.inv_depth_scale;
-          const float x = (u2f_exact((unsigned)u) - f.cx) * f.ifx * D, y = (u2f_exact((unsigned)vv) - f.cy) * f.ify * D;
-          const float px = R0 * x + R1 * y + R2 * D + t0;
-          const float py = R3 * x + R4 * y + R5 * D + t1;
-          const float pz = R6 * x + R7 * y + R8 * D + t2;
-          float V, gV[3], I, gI[3];
-          bool colour;
-          unsigned long long fresh = kEmpty;
-          const bool found = model_sample<ST>(d.v, p, px, py, pz, &V, gV, &I, gI, &colour, cj, &fresh);
-          if (fresh != kEmpty && d.pxcache) __stcg(d.pxcache + (size_t)vv * f.W + u, fresh);
-          if (!found) continue;
-          const float Jd[6] = {gV[0], gV[1], gV[2], py * gV[2] - pz * gV[1], pz * gV[0] - px * gV[2],
-                               px * gV[1] - py * gV[0]};
-          add_jtj(acc, Jd, V, 1.0f);
-          acc[28] += 1.0f;
-          if (colour) {
-            const float rc = I - rgb_intensity_raw(rgbj) * kIntensityScale;
-            const float Jc[6] = {gI[0], gI[1], gI[2], py * gI[2] - pz * gI[1], pz * gI[0] - px * gI[2],
-                                 px * gI[1] - py * gI[0]};
-            add_jtj(acc, Jc, rc, p.w_c);
+          if (r.z > 0.0f) {
+            const unsigned long long fresh = add_sample<ST>(d.v, c, pose, r.x, r.y, r.z, r.w, cj, acc);
+            if (fresh != kEmpty) d.pxcache[m.pixel(here)] = fresh;
           }
         }
         // chunk partial: a butterfly over the warp that halves the vector at
         // every step (31 shuffles for 32 slots) and leaves component c on
         // lane c, then the warps in fixed order
-        {
+        if (any) {
+          __syncwarp();
           float v[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] = i < 29 ? acc[i] : 0.0f;
+          for (int q = 0; q < 28; ++q) {
+            float a, b;
+            unpk(acc.v[q], a, b);
+            v[q] = a + b;
+          }
+          v[28] = acc.n;
+          v[29] = v[30] = v[31] = 0.0f;
 #pragma unroll
           for (int h = 16; h > 0; h >>= 1) {
             const bool upper = (lane & h) != 0;
 #pragma unroll
-            for (int i = 0; i < h; ++i) {
-              const float keep = upper ? v[i + h] : v[i];
-              const float send = upper ? v[i] : v[i + h];
-              v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+            for (int q = 0; q < h; ++q) {
+              const float keep = upper ? v[q + h] : v[q];
+              const float send = upper ? v[q] : v[q + h];
+              v[q] = keep + __shfl_xor_sync(0xffffffffu, send, h);
             }
           }
-          if (lane < 29) red[step & 1][warp][lane] = v[0];
+          red[step & 1][warp][lane] = v[0];
+        } else {
+          red[step & 1][warp][lane] = 0.0f;
         }
-        // the next step's pixels: loads issued now, used after the partials
-        pre = lb + G * slots * (step + 1) < nchunks;
-        if (pre) load_pixels(d, P, ch + G * slots, chunk, npix, nchunks, Ws, magic, stride, tin);
+        // the first record of the next step (or of the next evaluation, which
+        // samples the same pixels): the loads complete during the exchange
+        {
+          const bool more = lb + per_step * (step + 1) < nchunks;
+          const int j = bounds(more ? ch + per_step : lb + G * slot, end);
+          if (j < end) {
+            rec = d.rec[j];
+            cached = d.pxcache[m.pixel(j)];
+          }
+        }
         __syncthreads();
-        // the chunk partial of each slot: its warps' sums in order, tagged.
-        // No barrier after it: the next step writes the other buffer, and
-        // this one again only after the next step's barrier, which these
-        // reads precede.
-        if (warp < slots && lane < 29) {
-          const int cs = lb + G * (warp + slots * step);
+        // the chunk partial of each slot: its warps' sums in order; lane w < 10
+        // writes components 3 w .. 3 w + 2 with the tag.  No barrier after
+        // it: the next step writes the other buffer, and this one again only
+        // after the next step's barrier, which these reads precede.
+        if (warp < slots) {
+          const int cs = lb + G * warp + per_step * step;
           if (cs < nchunks) {
             const int wpc = width / 32;
             float sv = 0.0f;
             for (int w = 0; w < wpc; ++w) sv += red[step & 1][warp * wpc + w][lane];
-            st_relaxed_gpu_u64(part + lane * nchunks + cs, ((unsigned long long)tag << 32) | __float_as_uint(sv));
+            const unsigned s0 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane) & 31));
+            const unsigned s1 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 1) & 31));
+            const unsigned s2 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 2) & 31));
+            if (lane < kRegWords) st_relaxed_gpu_b128(part + lane * d.max_slots + cs, s0, s1, s2, tag);
           }
         }
       }
       // arrival: one relaxed count per CTA (other warps' partial stores may
       // still be on their way: the readers check the tags)
-      if (threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
-      // the next evaluation of this level samples the same pixels: their
-      // loads are issued now and complete while the CTA waits for the others
-      pre = it < iters;
-      if (pre) load_pixels(d, P, lb + G * slot, chunk, npix, nchunks, Ws, magic, stride, tin);
-      if (threadIdx.x == 0)
+      if (threadIdx.x == 0) {
+        red_relaxed_gpu_add(d.tags + 2, 1u);
         s_arrived = await_count(d.tags + 2, (unsigned)(eval + 1) * (unsigned)G + d.bar_extra, d.spin_limit);
+      }
+      // meanwhile: the next candidate should this one be rejected
+      if (warp == 1 && !first && !last) {
+        const bool stop = lm_candidate(S.sums[cur], reinterpret_cast<const float*>(S.pose[iT]),
+                                       reinterpret_cast<const float*>(S.plo[iT]),
+                                       d.c.lambda_pow[min(k + 1, kLambdaPow) + kLambdaPow], d.c.eps_t2f, d.c.eps_r2f,
+                                       reinterpret_cast<float*>(S.pose[iR]), reinterpret_cast<float*>(S.plo[iR]), lane);
+        if (lane == 0) S.stop[1] = stop;
+      }
       __syncthreads();
       if (!s_arrived) {
         if (threadIdx.x == 0) atomicOr(d.status, ST_BARRIER);
@@ -666,42 +722,44 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
         break;
       }
       // every CTA of the group: FP32 reduction of the chunk partials in a fixed
-      // order (lane-strided sums, then a shuffle tree); a word without this
-      // evaluation's tag is read again until it has it
+      // order (lane-strided sums, then a shuffle tree), one warp per word of
+      // three components; a word without this evaluation's tag is read again
+      // until it has it
       bool ok = true;
-      {
-        const int ca = warp, cb = warp + kRegWarps;  // warp w: components w and w + 16
-        const unsigned long long* ra = part + ca * nchunks;
-        const unsigned long long* rb = part + (cb < 29 ? cb : ca) * nchunks;
-        float fa = 0.0f, fb = 0.0f;
-        for (int k0 = lane; k0 < nchunks && ok; k0 += 32 * kReduceBatch) {
-          // the loads of a batch are issued together (one L2 round trip),
-          // then checked and added in order
-          unsigned long long va[kReduceBatch], vb[kReduceBatch];
+      float* sums = S.sums[cur ^ 1];
+      if (warp < kRegWords) {
+        const ulonglong2* row = part + warp * d.max_slots;
+        // all loads are issued together (one L2 round trip), then checked and
+        // added in order
+        constexpr int kLoads = (kRegChunks + 31) / 32;
+        ulonglong2 w[kLoads];
 #pragma unroll
-          for (int u = 0; u < kReduceBatch; ++u) {
-            const int k = k0 + 32 * u;
-            va[u] = k < nchunks ? ld_relaxed_gpu_u64(ra + k) : 0ull;
-            vb[u] = k < nchunks ? ld_relaxed_gpu_u64(rb + k) : 0ull;
-          }
+        for (int u = 0; u < kLoads; ++u) {
+          const int q = lane + 32 * u;
+          w[u] = make_ulonglong2(0ull, 0ull);
+          if (q < nchunks) w[u] = ld_relaxed_gpu_b128(row + q);
+        }
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
 #pragma unroll
-          for (int u = 0; u < kReduceBatch; ++u) {
-            const int k = k0 + 32 * u;
-            if (k < nchunks) {
-              ok = ok && await_tag(ra + k, va[u], tag, d.spin_limit) && await_tag(rb + k, vb[u], tag, d.spin_limit);
-              fa += __uint_as_float((unsigned)va[u]);
-              fb += __uint_as_float((unsigned)vb[u]);
-            }
+        for (int u = 0; u < kLoads; ++u) {
+          const int q = lane + 32 * u;
+          if (q < nchunks) {
+            ok = ok && await_tag(row + q, w[u], tag, d.spin_limit);
+            s0 += __uint_as_float((unsigned)w[u].x);
+            s1 += __uint_as_float((unsigned)(w[u].x >> 32));
+            s2 += __uint_as_float((unsigned)w[u].y);
           }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-          fa += __shfl_down_sync(0xffffffffu, fa, o);
-          fb += __shfl_down_sync(0xffffffffu, fb, o);
+          s0 += __shfl_down_sync(0xffffffffu, s0, o);
+          s1 += __shfl_down_sync(0xffffffffu, s1, o);
+          s2 += __shfl_down_sync(0xffffffffu, s2, o);
         }
         if (lane == 0) {
-          S.redf[ca] = fa;
-          if (cb < 29) S.redf[cb] = fb;
+          sums[3 * warp] = s0;
+          sums[3 * warp + 1] = s1;
+          sums[3 * warp + 2] = s2;
         }
       }
       if (!__syncthreads_and(ok)) {  // some wait ran out: leave, reporting it once per CTA
@@ -709,25 +767,83 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
         failed = true;
         break;
       }
-      if (warp == 0) lm_step_warp(S, mode, l, it == iters, d.c, lane);
+      // The LM step.  First evaluation of a level (at the accepted pose):
+      // always taken.  Later ones: the candidate is accepted when the mean
+      // cost decreases (En/Nn < E/N, compared exactly as En N < E Nn on the
+      // integer mantissas).
+      if (warp == 0 && !last) {
+        const int from = first ? iT : iC;
+        const int ka = first ? 0 : max(k - 1, -kLambdaPow);
+        const bool stop = lm_candidate(sums, reinterpret_cast<const float*>(S.pose[from]),
+                                       reinterpret_cast<const float*>(S.plo[from]), d.c.lambda_pow[ka + kLambdaPow],
+                                       d.c.eps_t2f, d.c.eps_r2f, reinterpret_cast<float*>(S.pose[iA]),
+                                       reinterpret_cast<float*>(S.plo[iA]), lane);
+        if (lane == 0) S.stop[0] = stop;
+      }
+      if (threadIdx.x == 32) {
+        const float En = sums[27];
+        const unsigned Nn = (unsigned)(sums[28] + 0.5f);  // below 2^24 as are the products' factors
+        const bool enough = (long long)Nn >= d.c.min_valid;
+        const bool accept = first || (enough && prod_less(En, S.N, S.E, Nn));
+        S.info.evals++;
+        S.info.level_evals[l]++;
+        if (accept) {
+          S.E = En;
+          S.N = Nn;
+          S.fin_E = En;
+          S.fin_N = Nn;
+        }
+        S.accept = accept ? (first && !enough ? 2 : 1) : 0;  // 2: too few pixels, the level ends
+      }
       __syncthreads();
       ++eval;
+      // every thread follows the decision: slots and damping
+      const int accept = S.accept;
+      if (accept) {
+        cur ^= 1;
+        if (first) {
+          k = 0;
+          const int t = iC;  // the candidate slot is free: the next candidate takes it
+          iC = iA;
+          iA = t;
+        } else {
+          k = max(k - 1, -kLambdaPow);
+          moved = true;
+          const int t = iT;
+          iT = iC;
+          iC = iA;
+          iA = t;
+        }
+      } else {
+        k = min(k + 1, kLambdaPow);
+        const int t = iC;
+        iC = iR;
+        iR = t;
+      }
+      if (accept == 2) {
+        done = true;
+      } else if (!last && S.stop[accept ? 0 : 1]) {
+        done = true;
+        if (threadIdx.x == 0) S.info.converged[l] = 1;
+      }
     }
   }
-  leave_registration(d, lb, G, tag0);
+  leave_registration(d, G, tag0);
   if (failed) return;
   if (lb == 0) {
     if (threadIdx.x < 16) {  // the pose in FP64: hi + lo of each entry, the last row 0 0 0 1
-      const int i = threadIdx.x >> 2, j = threadIdx.x & 3;
-      const int fi = j < 3 ? i * 3 + j : 9 + i;
-      d.T_out[threadIdx.x] = i == 3   ? (j == 3 ? 1.0 : 0.0)
-                             : S.moved ? (double)S.Rf[fi] + (double)S.Rlf[fi]
-                                       : S.T0[fi];
+      const int q = threadIdx.x;
+      double t = q == 15 ? 1.0 : 0.0;
+      if (q < 12)
+        t = moved ? (double)reinterpret_cast<const float*>(S.pose[iT])[q] +
+                        (double)reinterpret_cast<const float*>(S.plo[iT])[q]
+                  : S.T0[q];
+      d.T_out[q] = t;
     }
     if (threadIdx.x == 0 && d.info) {
       rf_track_info out = S.info;
-      out.final_cost = S.fin_N > 0 ? (double)S.fin_E / (double)S.fin_N : 0.0;
-      out.final_valid = S.fin_N;
+      out.final_cost = S.fin_N > 0u ? (double)S.fin_E / (double)S.fin_N : 0.0;
+      out.final_valid = (int64_t)S.fin_N;
       *d.info = out;
     }
   }
@@ -799,6 +915,7 @@ RegDesc make_reg_desc(rf_volume* vol, const DevFrame& f, const double* T_init, c
   d.spin_limit = vol->wait_spins;
   d.bar_extra = vol->wait_extra;
   d.pxcache = vol->d_pxcache;
+  d.rec = reinterpret_cast<float4*>(vol->d_cand);
   return d;
 }
 

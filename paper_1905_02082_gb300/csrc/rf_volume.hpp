@@ -33,11 +33,11 @@ struct rf_volume {
   unsigned* d_status = nullptr;
 
   // registration scratch
-  // 2 x 29 x max_slots tagged partial sums of the registration (tag << 32 |
-  // float bits).  Mesh extraction and virtual-depth filling reuse word 0 as a
-  // counter between registrations: a count below 2^32 in it, or in its low
-  // half, leaves a tag no later registration waits for.
-  unsigned long long* d_partials = nullptr;
+  // 2 x kRegWords x max_slots tagged partial sums of the registration (three
+  // floats, then the tag in the top 32 bits of each 16-byte word).  Mesh
+  // extraction and virtual-depth filling reuse the first 8 bytes as a counter
+  // between registrations: they are below the first word's tag.
+  ulonglong2* d_partials = nullptr;
   int max_slots = 0;
   unsigned* d_regtags = nullptr;  // registration tag base and leaving count
   int reg_grid = 0;
@@ -52,7 +52,7 @@ struct rf_volume {
   rf::IntegState* d_integ = nullptr;
   int* d_tilemax = nullptr;
   uint16_t* d_dmask = nullptr;  // per pixel: raw depth if valid and not masked, else 0
-  int4* d_cand = nullptr;
+  int4* d_cand = nullptr;  // also the registration's pixel records (max_candidates or max_w * max_h entries, the larger)
 
   // whole-frame staging (graph-replayed pipeline reads only these)
   uint16_t* d_depth = nullptr;
