@@ -145,6 +145,16 @@ rf_status check_volume_args(const rf_params* p, int64_t n_buckets, int64_t max_b
 // kRegChunks of them).
 size_t reg_slots(size_t npix) { return std::min<size_t>(kRegChunks, (npix + 127) / 128); }
 
+// Pixel records of a registration: the sampled pixels of its three levels.
+size_t reg_records(const rf_params* p, int w, int h) {
+  size_t n = 0;
+  for (int l = 0; l < 3; ++l) {
+    const int s = p->lm_strides[l];
+    n += (size_t)((w + s - 1) / s) * ((h + s - 1) / s);
+  }
+  return n;
+}
+
 // Every device buffer of a volume, in one list: rf_create_volume allocates
 // them, rf_volume_footprint adds up their sizes.
 template <class Alloc>
@@ -166,7 +176,7 @@ rf_status volume_buffers(rf_volume* vol, const rf_params* p, int64_t n_buckets, 
       (s = A(&vol->d_dmask, npix, "masked depth")) ||
       // (a registration keeps its pixel records in the candidate list's memory:
       // the two never run at the same time on one volume)
-      (s = A(&vol->d_cand, std::max((size_t)p->max_candidates, npix), "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
+      (s = A(&vol->d_cand, std::max((size_t)p->max_candidates, reg_records(p, max_width, max_height)), "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
       (s = A(&vol->d_rgb, npix * 3, "rgb staging")) || (s = A(&vol->d_mask, npix, "mask staging")) ||
       (s = A(&vol->d_T, 48, "poses")) || (s = A(&vol->d_info, 1, "info")) || (s = A(&vol->d_guard, 1, "guard count")) ||
       (s = A(&vol->d_pxcache, npix, "pixel block cache")))
@@ -681,7 +691,7 @@ rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_bl
   const size_t npix = (size_t)max_width * max_height;
   vol->max_slots = (int)reg_slots(npix);
   vol->reg_grid = register_max_grid(vol->device);
-  if (vol->reg_grid > vol->sm_count) vol->reg_grid = vol->sm_count;
+  vol->reg_grid = std::min(vol->reg_grid, vol->sm_count);
   if (vol->reg_grid < 1) {
     s = set_error(nullptr, RF_ERR_CUDA, "registration kernel cannot be resident on this device");
     delete vol;

@@ -134,8 +134,8 @@ struct RegDesc {
   // was found in, ~0 when none; a block's pool never changes until the
   // volume is reset or imported, which clear the cache
   unsigned long long* pxcache;
-  // per sampled pixel of the current level: camera point and scaled
-  // intensity, written and read by the thread that samples it
+  // per sampled pixel of each level: camera point and scaled intensity,
+  // written and read by the thread that samples it
   float4* rec;
 };
 
@@ -435,6 +435,7 @@ __device__ __forceinline__ void st_relaxed_gpu_b128(ulonglong2* p, unsigned a, u
                "l"(lo), "l"(hi)
                : "memory");
 }
+
 __device__ __forceinline__ void red_relaxed_gpu_add(unsigned* p, unsigned v) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -447,19 +448,6 @@ __device__ __forceinline__ bool await_count(const unsigned* count, unsigned targ
   while (ld_relaxed_gpu(count) < target) {
     if (++spins > spin_limit) return false;
     if (spins > 4096) __nanosleep(64);
-  }
-  return true;
-}
-
-// Waits until the tagged word *p (last read into v) carries tag `want`,
-// re-polling at most spin_limit times (the same schedule); false when the
-// wait ran out.
-__device__ __forceinline__ bool await_tag(const ulonglong2* p, ulonglong2& v, unsigned want, long long spin_limit) {
-  long long spins = 0;
-  while ((unsigned)(v.y >> 32) != want) {
-    if (++spins > spin_limit) return false;
-    if (spins > 4096) __nanosleep(64);
-    v = ld_relaxed_gpu_b128(p);
   }
   return true;
 }

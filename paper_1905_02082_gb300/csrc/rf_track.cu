@@ -4,9 +4,9 @@
 // over three pixel sub-samplings (strides), coarse to fine.
 //
 // A whole registration (three levels, every LM iteration) is ONE cooperative
-// launch of k_register, one CTA of 512 threads per SM.  At the start of a
-// level every thread writes the records of its sampled pixels (camera point
-// and intensity) into a per-volume buffer that only it reads again.  Per cost
+// launch of k_register, one CTA of 512 threads per SM.  At its start every
+// thread writes the records of the pixels it will sample (camera point and
+// intensity) into a per-volume buffer that only it reads again.  Per cost
 // evaluation:
 //   1. every thread takes its pixels' records: rigid transform, hash lookup of
 //      the 8 lattice corners, trilinear SDF and intensity with analytic
@@ -22,10 +22,13 @@
 //      update lambda, solve the damped 6x6 system and compose the next
 //      candidate pose exp(delta) T (FP32 with exactly formed residuals and a
 //      pose carried as float pairs; see lm_candidate).  Identical inputs and
-//      code give identical states in all CTAs, so no broadcast is needed.
-// The LM state never leaves shared memory; a level ends early when the step
-// falls below the thresholds.  Results are deterministic: fixed chunks, fixed
-// pixel-to-thread mapping, fixed reduction order.
+//      code give identical states in all CTAs, so no broadcast is needed: a
+//      second hop through L2 costs more than the redundant step (one CTA
+//      running the step and sending the pose to the others was measured at
+//      123 us a 640x480 registration, this form at 102).
+// A level ends early when the step falls below the thresholds.  Results are
+// deterministic: fixed chunks, fixed pixel-to-thread mapping, fixed reduction
+// order.
 #include <cmath>
 #include <type_traits>
 
@@ -71,6 +74,12 @@ struct Acc {
   f2 v[28];
   float n;
 };
+
+__device__ __forceinline__ void clear(Acc& acc) {
+#pragma unroll
+  for (int i = 0; i < 28; ++i) acc.v[i] = 0ull;
+  acc.n = 0.0f;
+}
 
 // The per-sample constants of a registration (uniform over the CTA).
 struct SampleConst {
@@ -213,9 +222,16 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
   J[0] = gx;
   J[1] = gy;
   J[2] = gz;
-  J[3] = fma2(pk(py, py), gz, mul2(pk(-pz, -pz), gy));
-  J[4] = fma2(pk(pz, pz), gx, mul2(pk(-px, -px), gz));
-  J[5] = fma2(pk(px, px), gy, mul2(pk(-py, -py), gx));
+  {
+    // p x g, one half at a time: packing p twice costs more than it saves
+    float ax, ay, az, bx, by, bz;
+    unpk(gx, ax, bx);
+    unpk(gy, ay, by);
+    unpk(gz, az, bz);
+    J[3] = pk(fmaf(py, az, -pz * ay), fmaf(py, bz, -pz * by));
+    J[4] = pk(fmaf(pz, ax, -px * az), fmaf(pz, bx, -px * bz));
+    J[5] = pk(fmaf(px, ay, -py * ax), fmaf(px, by, -py * bx));
+  }
   int n = 0;
 #pragma unroll
   for (int i = 0; i < 6; ++i)
@@ -231,21 +247,29 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
   return fresh;
 }
 
-// LM state of one registration, one copy in the shared memory of every CTA.
-// Poses are kept as pairs of floats per entry (hi + lo, about 48 bits; hi is
-// the float pose an evaluation uses), rows (R | t) of four.
-struct LMShared {
-  float sums[2][32];    // FP32 sums of an evaluation: 21 of J^T J, 6 of J^T r, cost, valid count; one slot holds the
-                        // accepted pose's, the other the evaluation just reduced
-  float4 pose[4][3];    // hi parts: the accepted pose, the candidate, and the two possible next candidates
-  float4 plo[4][3];     // lo parts
-  int stop[2];          // next candidate after an acceptance / a rejection: 1 when there is none (level converged)
+// Geometry of one level: sampled pixels Ws x Hs, `chunk` of them per partial
+// sum, and where its records start in the record buffer.
+struct Level {
+  int Ws, stride, npix, chunk, nchunks, rec0;
+  unsigned long long magic;  // ceil(2^32 / Ws)
+};
+
+// State of a registration, one copy in the shared memory of every CTA.  Poses
+// are rows (R | t) of four, as pairs of floats per entry (hi + lo, about 48
+// bits; hi is the float pose an evaluation uses).
+struct RegShared {
+  Level level[3];
+  int arrived;
+  float sums[2][32];  // FP32 sums of an evaluation: 21 of J^T J, 6 of J^T r, cost, valid count; one slot holds the
+                      // accepted pose's, the other the evaluation just reduced
+  float4 pose[4][3];  // hi parts: the accepted pose, the candidate, and the two possible next candidates
+  float plo[4][12];   // lo parts
+  int stop[2][2];     // by parity of the evaluation: 1 when there is no next candidate (level converged) after an
+                      // acceptance / a rejection
   int accept;
-  float E;              // cost and valid count of the accepted pose
+  float E;            // cost and valid count of the accepted pose
   unsigned N;
-  float fin_E;
-  unsigned fin_N;
-  double T0[12];        // the initial pose, returned unchanged when no candidate is accepted
+  double T0[12];      // the initial pose, returned unchanged when no candidate is accepted
   rf_track_info info;
 };
 
@@ -253,6 +277,12 @@ struct LMShared {
 // 6x6 matrix (row-major: the order of the 21 sums of J^T J).
 __host__ __device__ constexpr int up6(int i, int j) { return i * 6 - i * (i - 1) / 2 + (j - i); }
 
+
+__device__ __forceinline__ float rsqrt_approx(float x) {  // normal x
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 
 // FP32 Cholesky factorisation of the damped matrix in place: A holds the
 // upper triangle (row-major) on entry and L^T (L's column j stored as row j of
@@ -268,7 +298,7 @@ __device__ __forceinline__ bool chol6(float A[21], float inv[6]) {
   for (int j = 0; j < 6; ++j) {
     const float s = A[up6(j, j)];
     ok = ok && (s > 0.0f) && (s < 3.0e38f);
-    const float r = rsqrtf(fmaxf(s, 1.0e-30f));
+    const float r = rsqrt_approx(fmaxf(s, 1.0e-30f));
     A[up6(j, j)] = s * r;
     inv[j] = r;
 #pragma unroll
@@ -365,25 +395,28 @@ __device__ __noinline__ bool lm_candidate(const float* sums, const float* hi, co
   const bool ok = chol6(A, inv);
   chol6_solve(A, inv, d);
   // residual -g - (H + lambda diag H) d, exact to about 2^-46: row i on
-  // lane i, then gathered on every lane
+  // lane i, then gathered on every lane.  No branches (a divergent one per
+  // column made this 1,000 of the step's 2,500 cycles): the damping term
+  // lambda h_ii d_i is a seventh product.
   {
     const int i = lane < 6 ? lane : 0;
-    float sh = -sums[21 + i], sl = 0.0f;
+    const int row = up6(i, i) - i;  // entry (i, j), j >= i, at row + j
+    float sh = -sums[21 + i], sl = 0.0f, hii = 0.0f, di = 0.0f;
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const float h = sums[i <= j ? up6(i, j) : up6(j, i)];
+      const float h = sums[i <= j ? row + j : up6(j, j) - j + i];
+      hii = i == j ? h : hii;
+      di = i == j ? d[j] : di;
       float p, pe, e;
       two_prod(h, d[j], p, pe);
       two_sum(sh, -p, sh, e);
       sl += e - pe;
-      if (i == j) {  // the damping term lambda h d
-        float lh, lhe;
-        two_prod(lam, h, lh, lhe);
-        two_prod(lh, d[j], p, pe);
-        two_sum(sh, -p, sh, e);
-        sl += e - pe - lhe * d[j];
-      }
     }
+    float lh, lhe, p, pe, e;
+    two_prod(lam, hii, lh, lhe);
+    two_prod(lh, di, p, pe);
+    two_sum(sh, -p, sh, e);
+    sl += e - pe - lhe * di;
     const float ri = sh + sl;
 #pragma unroll
     for (int q = 0; q < 6; ++q) r[q] = __shfl_sync(0xffffffffu, ri, q);
@@ -413,30 +446,32 @@ __device__ __noinline__ bool lm_candidate(const float* sums, const float* hi, co
   // carried as float pairs (lanes 0-11: rows 0-2, columns 0-3).  Row i of
   // exp(d) - I: Er = A K + B K^2 with K v = phi x v and K^2 = phi phi^T -
   // theta^2 I; et = rho + B K rho + C K^2 rho.
+  const int at = lane < 12 ? lane : 0;
+  const int i = at >> 2, j = at & 3;
+  const float h0 = hi[j], h1 = hi[4 + j], h2 = hi[8 + j], hT = hi[at], lT = lo[at];
+  const float pi = i == 0 ? p0 : (i == 1 ? p1 : p2);
+  // row i of K: (K_i0, K_i1, K_i2)
+  const float k0 = i == 0 ? 0.0f : (i == 1 ? p2 : -p1);
+  const float k1 = i == 0 ? -p2 : (i == 1 ? 0.0f : p0);
+  const float k2 = i == 0 ? p1 : (i == 1 ? -p0 : 0.0f);
+  const float e0 = fmaf(cA, k0, cB * fmaf(pi, p0, i == 0 ? -t2 : 0.0f));
+  const float e1 = fmaf(cA, k1, cB * fmaf(pi, p1, i == 1 ? -t2 : 0.0f));
+  const float e2 = fmaf(cA, k2, cB * fmaf(pi, p2, i == 2 ? -t2 : 0.0f));
+  float inc = fmaf(e0, h0, fmaf(e1, h1, e2 * h2));
+  // column 3: + (rho + B K rho + C K^2 rho)_i
+  const float kr = fmaf(k0, d[0], fmaf(k1, d[1], k2 * d[2]));  // (K rho)_i
+  const float kr0 = p1 * d[2] - p2 * d[1], kr1 = p2 * d[0] - p0 * d[2], kr2 = p0 * d[1] - p1 * d[0];
+  const float kk = fmaf(k0, kr0, fmaf(k1, kr1, k2 * kr2));  // (K K rho)_i
+  const float rho_i = i == 0 ? d[0] : (i == 1 ? d[1] : d[2]);
+  const float trans = fmaf(cC, kk, fmaf(cB, kr, rho_i));
+  inc += j == 3 ? trans : 0.0f;
+  float sum, err;
+  two_sum(hT, inc, sum, err);
+  err += lT;
+  const float hn = sum + err;  // renormalised: hn is the nearest float of the pair's sum
   if (lane < 12) {
-    const int i = lane >> 2, j = lane & 3;
-    const float pi = i == 0 ? p0 : (i == 1 ? p1 : p2);
-    // row i of K: (K_i0, K_i1, K_i2)
-    const float k0 = i == 0 ? 0.0f : (i == 1 ? p2 : -p1);
-    const float k1 = i == 0 ? -p2 : (i == 1 ? 0.0f : p0);
-    const float k2 = i == 0 ? p1 : (i == 1 ? -p0 : 0.0f);
-    const float e0 = fmaf(cA, k0, cB * fmaf(pi, p0, i == 0 ? -t2 : 0.0f));
-    const float e1 = fmaf(cA, k1, cB * fmaf(pi, p1, i == 1 ? -t2 : 0.0f));
-    const float e2 = fmaf(cA, k2, cB * fmaf(pi, p2, i == 2 ? -t2 : 0.0f));
-    float inc = fmaf(e0, hi[j], fmaf(e1, hi[4 + j], e2 * hi[8 + j]));
-    if (j == 3) {  // + (rho + B K rho + C K^2 rho)_i
-      const float kr = fmaf(k0, d[0], fmaf(k1, d[1], k2 * d[2]));  // (K rho)_i
-      const float kr0 = p1 * d[2] - p2 * d[1], kr1 = p2 * d[0] - p0 * d[2], kr2 = p0 * d[1] - p1 * d[0];
-      const float kk = fmaf(k0, kr0, fmaf(k1, kr1, k2 * kr2));  // (K K rho)_i
-      const float rho_i = i == 0 ? d[0] : (i == 1 ? d[1] : d[2]);
-      inc += fmaf(cC, kk, fmaf(cB, kr, rho_i));
-    }
-    float sum, err;
-    two_sum(hi[lane], inc, sum, err);
-    err += lo[lane];
-    const float h2 = sum + err;  // renormalised: h2 is the nearest float of the pair's sum
-    out[lane] = h2;
-    out_lo[lane] = err - (h2 - sum);
+    out[lane] = hn;
+    out_lo[lane] = err - (hn - sum);
   }
   return false;
 }
@@ -454,34 +489,30 @@ __device__ __forceinline__ int chunk_pixels(int npix) {
   return max(128, (c + 127) & ~127);
 }
 
-// Pixel index in the frame of sample i of a level (row = i / Ws by a
-// reciprocal multiply, off by at most one for i < 2^32, then corrected).
-struct LevelMap {
-  int Ws, stride, W;
-  unsigned long long magic;
-  __device__ __forceinline__ void locate(int i, int& u, int& v) const {
-    int row = (int)(((unsigned long long)i * magic) >> 32);
-    if (row * Ws > i) --row;
-    else if ((row + 1) * Ws <= i) ++row;
-    u = (i - row * Ws) * stride;
-    v = row * stride;
-  }
-  __device__ __forceinline__ int pixel(int i) const {
-    if (stride == 1) return i;
-    int u, v;
-    locate(i, u, v);
-    return v * W + u;
-  }
-};
+// Position in the frame of sample i of a level (row = i / Ws by a reciprocal
+// multiply, off by at most one for i < 2^32, then corrected).
+__device__ __forceinline__ void locate(const Level& L, int i, int& u, int& v) {
+  int row = (int)(((unsigned long long)i * L.magic) >> 32);
+  if (row * L.Ws > i) --row;
+  else if ((row + 1) * L.Ws <= i) ++row;
+  u = (i - row * L.Ws) * L.stride;
+  v = row * L.stride;
+}
+__device__ __forceinline__ int pixel_of_sample(const Level& L, int W, int i) {
+  if (L.stride == 1) return i;
+  int u, v;
+  locate(L, i, u, v);
+  return v * W + u;
+}
 
-// Record of sample i of a level, written once per level by the thread that
-// samples it: camera point of Eq. 1 and minus sqrt(w_c) times the intensity;
-// z = 0 where the pixel is not sampled (invalid depth or masked).
-__device__ __forceinline__ void write_record(const RegDesc& d, const LevelMap& m, float col_off, int i) {
+// Record of sample i of a level, written once per registration by the thread
+// that samples it: camera point of Eq. 1 and minus sqrt(w_c) times the
+// intensity; z = 0 where the pixel is not sampled (invalid depth or masked).
+__device__ __forceinline__ void write_record(const RegDesc& d, const Level& L, float col_off, int i) {
   const DevFrame& f = d.f;
   int u, v;
-  m.locate(i, u, v);
-  const int idx = v * m.W + u;
+  locate(L, i, u, v);
+  const int idx = v * f.W + u;
   unsigned raw = __ldg(f.depth + idx);
   if (d.mask && __ldg(d.mask + idx)) raw = 0u;
   const uint8_t* cp = f.rgb + 3 * (size_t)idx;
@@ -494,12 +525,12 @@ __device__ __forceinline__ void write_record(const RegDesc& d, const LevelMap& m
     r.z = D;
     r.w = rgb_intensity_raw(rgb) * col_off;
   }
-  d.rec[i] = r;
+  d.rec[L.rec0 + i] = r;
 }
 
-// Every CTA of a registration group calls this once, after its last read of
-// the partial sums.  The last CTA to leave clears the arrival count and
-// advances the tag base past the
+// Every CTA of a registration group calls this once, after its last use of
+// the exchange.  The last CTA to leave clears the arrival count and advances
+// the tag base past the
 // registration's tags (at most 3 + the sum of the level iteration caps); when
 // the tags would reach kTagLimit it first clears the whole partial buffer,
 // whose tags then all read 0, and restarts the base at 0.  Either way every
@@ -536,31 +567,49 @@ __device__ __forceinline__ void leave_registration(const RegDesc& d, int G, unsi
 // evaluation parity safe: a CTA writes evaluation e + 2 only after all G CTAs
 // arrived at e + 1, each after it had read all of evaluation e.
 //
-// The LM step is split over two warps so that little of it follows the
-// reduction: while the CTA waits for the others, warp 1 computes the next
-// candidate of a rejection (it needs the accepted pose's sums only); after
-// the reduction warp 0 computes the next candidate of an acceptance while
-// warp 1 decides which of the two applies.
+// Little of the LM step follows the reduction: while the CTA waits for the
+// others, one of its warps computes the next candidate of a rejection (it
+// needs the accepted pose's sums only); after the reduction warp 0 computes
+// the next candidate of an acceptance while another warp decides which of the
+// two applies.  The first of them shares warp 0's scheduler and so leaves its
+// instruction cache holding the step's code.
 template <int ST>
 __device__ void register_body(const RegDesc& d, int lb, int G) {
-  __shared__ LMShared S;
+  __shared__ RegShared S;
   __shared__ float red[2][kRegWarps][32];  // per-warp sums of a chunk, double-buffered by step parity
-  __shared__ int s_arrived;
+  constexpr int kRejectWarp = 12, kDecideWarp = 13;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const DevFrame& f = d.f;
 
-  if (threadIdx.x == 0) {
-    S.fin_E = 0.0f;
-    S.fin_N = 0u;
+  if (threadIdx.x < 3) {
+    const int l = threadIdx.x;
+    int rec0 = 0;
+    Level L;
+    for (int i = 0; i <= l; ++i) {
+      L.rec0 = rec0;
+      L.stride = d.c.strides[i];
+      L.Ws = (f.W + L.stride - 1) / L.stride;
+      L.npix = L.Ws * ((f.H + L.stride - 1) / L.stride);
+      rec0 += L.npix;
+    }
+    L.chunk = chunk_pixels(L.npix);
+    L.nchunks = (L.npix + L.chunk - 1) / L.chunk;
+    L.magic = (0x100000000ull + L.Ws - 1) / L.Ws;
+    S.level[l] = L;
+  }
+  if (threadIdx.x == 32) {
     rf_track_info z = {};
     S.info = z;
+    S.E = 0.0f;
+    S.N = 0u;
   }
-  if (threadIdx.x < 12) {  // the initial pose as float pairs (FP64 once per registration)
-    const double t = d.T_init[threadIdx.x];
-    S.T0[threadIdx.x] = t;
+  if (threadIdx.x >= 64 && threadIdx.x < 76) {  // the initial pose as float pairs (FP64 once per registration)
+    const int q = threadIdx.x - 64;
+    const double t = d.T_init[q];
+    S.T0[q] = t;
     const float hi = (float)t;
-    reinterpret_cast<float*>(S.pose[0])[threadIdx.x] = hi;
-    reinterpret_cast<float*>(S.plo[0])[threadIdx.x] = (float)(t - (double)hi);
+    reinterpret_cast<float*>(S.pose[0])[q] = hi;
+    S.plo[0][q] = (float)(t - (double)hi);
   }
   SampleConst c;
   {
@@ -571,62 +620,69 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
     c.col_scale = (ST == RF_STORAGE_FP32 ? kIntensityScale : kI8Scale) * swc;
     c.gs_col = c.col_scale * d.p.inv_voxel;
   }
-  const float col_off = -kIntensityScale * sqrtf(d.p.w_c);
   __syncthreads();
   const unsigned tag0 = ld_relaxed_gpu(d.tags);  // written by the previous registration's last CTA
-  int eval = 0;
+
+  // chunks narrower than the CTA run side by side, one per warp group (slot):
+  // chunk lb + G (slot + slots step) at each step
+  int chunk = 0, nchunks = 0, npix = 0, width = 1, slots = 1, slot = 0, tin = 0;
+  auto set_level = [&](const Level& L) {
+    chunk = L.chunk;
+    nchunks = L.nchunks;
+    npix = L.npix;
+    width = min(chunk, kRegThreads);  // threads per chunk
+    slots = kRegThreads / width;
+    slot = threadIdx.x / width;
+    tin = threadIdx.x - slot * width;
+  };
+  // this thread's samples of a chunk: first, first + width, ... below end
+  auto bounds = [&](int ch, int& end) {
+    end = slot < slots && ch < nchunks ? min(npix, (ch + 1) * chunk) : 0;
+    return ch * chunk + tin;
+  };
+  {
+    const float col_off = -kIntensityScale * sqrtf(d.p.w_c);
+    for (int l = 0; l < 3; ++l) {
+      set_level(S.level[l]);
+      for (int ch = lb + G * slot; ch < nchunks && slot < slots; ch += G * slots) {
+        int end;
+        for (int i = bounds(ch, end); i < end; i += width) write_record(d, S.level[l], col_off, i);
+      }
+    }
+  }
+
+  unsigned eval = 0;
   bool failed = false, moved = false;
   int iT = 0, iC = 1, iA = 2, iR = 3;  // pose slots: accepted, candidate, next after acceptance, next after rejection
   int cur = 0;                         // slot of S.sums that holds the accepted pose's
+  Acc acc;                             // empty between the steps
+  clear(acc);
   for (int l = 0; l < 3 && !failed; ++l) {
-    LevelMap m;
-    m.stride = d.c.strides[l];
-    m.W = f.W;
-    m.Ws = (f.W + m.stride - 1) / m.stride;
-    m.magic = (0x100000000ull + m.Ws - 1) / m.Ws;
-    const int npix = m.Ws * ((f.H + m.stride - 1) / m.stride);
-    const int chunk = chunk_pixels(npix);
-    const int nchunks = (npix + chunk - 1) / chunk;
+    const Level& L = S.level[l];
+    const float4* records = d.rec + L.rec0;
+    set_level(L);
     const int iters = d.c.iters[l];
-    // chunks narrower than the CTA run side by side, one per warp group
-    // (slot): chunk lb + G (slot + slots step) at each step
-    const int width = min(chunk, kRegThreads);  // threads per chunk
-    const int slots = kRegThreads / width;
-    const int slot = threadIdx.x / width, tin = threadIdx.x - slot * width;
-    const int per_step = G * slots;
-    // this thread's samples of a chunk: first, first + width, ... below end
-    auto bounds = [&](int ch, int& end) {
-      end = slot < slots && ch < nchunks ? min(npix, (ch + 1) * chunk) : 0;
-      return ch * chunk + tin;
-    };
-    for (int ch = lb + G * slot; ch < nchunks && slot < slots; ch += per_step) {
-      int end;
-      for (int i = bounds(ch, end); i < end; i += width) write_record(d, m, col_off, i);
-    }
-    bool done = false;
-    int k = 0;  // damping lambda0 10^k: rejections minus acceptances
-    // the first sample's record of the next evaluation, loaded ahead of it
+    // the next sample's record and cached block entry
     float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     unsigned long long cached = kEmpty;
+    auto fetch = [&](int i) {
+      rec = records[i];
+      cached = d.pxcache[pixel_of_sample(L, f.W, i)];
+    };
     {
       int end;
       const int i = bounds(lb + G * slot, end);
-      if (i < end) {
-        rec = d.rec[i];
-        cached = d.pxcache[m.pixel(i)];
-      }
+      if (i < end) fetch(i);
     }
+    bool done = false;
+    int k = 0;  // damping lambda0 10^k: rejections minus acceptances
     for (int it = 0; it <= iters && !done; ++it) {
       const bool first = it == 0, last = it == iters;
       const float4* pose = S.pose[first ? iT : iC];
-      ulonglong2* part = d.partials + (size_t)(eval & 1) * kRegWords * d.max_slots;
-      const unsigned tag = tag0 + (unsigned)eval + 1u;
-      for (int step = 0; lb + per_step * step < nchunks; ++step) {
-        const int ch = lb + G * slot + per_step * step;
-        Acc acc;
-#pragma unroll
-        for (int i = 0; i < 28; ++i) acc.v[i] = 0ull;
-        acc.n = 0.0f;
+      ulonglong2* part = d.partials + (size_t)(eval & 1u) * kRegWords * d.max_slots;
+      const unsigned tag = tag0 + eval + 1u;
+      for (int step = 0; lb + G * slots * step < nchunks; ++step) {
+        const int ch = lb + G * (slot + slots * step);
         int end;
         int i = bounds(ch, end);
         const bool any = __any_sync(0xffffffffu, i < end);
@@ -636,18 +692,16 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
           const unsigned long long cj = cached;
           const int here = i;
           i += width;
-          if (i < end) {  // the next sample's record
-            rec = d.rec[i];
-            cached = d.pxcache[m.pixel(i)];
-          }
+          if (i < end) fetch(i);  // the next sample's record
           if (r.z > 0.0f) {
             const unsigned long long fresh = add_sample<ST>(d.v, c, pose, r.x, r.y, r.z, r.w, cj, acc);
-            if (fresh != kEmpty) d.pxcache[m.pixel(here)] = fresh;
+            if (fresh != kEmpty) d.pxcache[pixel_of_sample(L, f.W, here)] = fresh;
           }
         }
         // chunk partial: a butterfly over the warp that halves the vector at
         // every step (31 shuffles for 32 slots) and leaves component c on
         // lane c, then the warps in fixed order
+        float* mine = &red[step & 1][warp][lane];
         if (any) {
           __syncwarp();
           float v[32];
@@ -669,82 +723,83 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
               v[q] = keep + __shfl_xor_sync(0xffffffffu, send, h);
             }
           }
-          red[step & 1][warp][lane] = v[0];
+          *mine = v[0];
         } else {
-          red[step & 1][warp][lane] = 0.0f;
-        }
-        // the first record of the next step (or of the next evaluation, which
-        // samples the same pixels): the loads complete during the exchange
-        {
-          const bool more = lb + per_step * (step + 1) < nchunks;
-          const int j = bounds(more ? ch + per_step : lb + G * slot, end);
-          if (j < end) {
-            rec = d.rec[j];
-            cached = d.pxcache[m.pixel(j)];
-          }
+          *mine = 0.0f;
         }
         __syncthreads();
         // the chunk partial of each slot: its warps' sums in order; lane w < 10
         // writes components 3 w .. 3 w + 2 with the tag.  No barrier after
         // it: the next step writes the other buffer, and this one again only
         // after the next step's barrier, which these reads precede.
-        if (warp < slots) {
-          const int cs = lb + G * warp + per_step * step;
-          if (cs < nchunks) {
-            const int wpc = width / 32;
-            float sv = 0.0f;
-            for (int w = 0; w < wpc; ++w) sv += red[step & 1][warp * wpc + w][lane];
-            const unsigned s0 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane) & 31));
-            const unsigned s1 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 1) & 31));
-            const unsigned s2 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 2) & 31));
-            if (lane < kRegWords) st_relaxed_gpu_b128(part + lane * d.max_slots + cs, s0, s1, s2, tag);
-          }
+        const int cs = lb + G * (warp + slots * step);
+        if (warp < slots && cs < nchunks) {
+          const int wpc = width / 32;
+          const float* from = &red[step & 1][warp * wpc][lane];
+          float t[kRegWarps], sv = 0.0f;
+#pragma unroll
+          for (int w = 0; w < kRegWarps; ++w) t[w] = w < wpc ? from[32 * w] : 0.0f;
+#pragma unroll
+          for (int w = 0; w < kRegWarps; ++w) sv += t[w];
+          const unsigned s0 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane) & 31));
+          const unsigned s1 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 1) & 31));
+          const unsigned s2 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 2) & 31));
+          if (lane < kRegWords) st_relaxed_gpu_b128(part + lane * d.max_slots + cs, s0, s1, s2, tag);
         }
+        const bool more = lb + G * slots * (step + 1) < nchunks;
+        // arrival: one relaxed count per CTA (other warps' partial stores may
+        // still be on their way: the readers check the tags)
+        if (!more && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
+        // for the next step (or the next evaluation, which samples the same
+        // pixels), during the exchange: empty sums and the first record
+        clear(acc);
+        const int j = bounds(more ? ch + G * slots : lb + G * slot, end);
+        if (j < end) fetch(j);
       }
-      // arrival: one relaxed count per CTA (other warps' partial stores may
-      // still be on their way: the readers check the tags)
-      if (threadIdx.x == 0) {
-        red_relaxed_gpu_add(d.tags + 2, 1u);
-        s_arrived = await_count(d.tags + 2, (unsigned)(eval + 1) * (unsigned)G + d.bar_extra, d.spin_limit);
-      }
+      if (lb >= nchunks && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
+      if (threadIdx.x == 0)
+        S.arrived = await_count(d.tags + 2, (eval + 1u) * (unsigned)G + d.bar_extra, d.spin_limit);
       // meanwhile: the next candidate should this one be rejected
-      if (warp == 1 && !first && !last) {
-        const bool stop = lm_candidate(S.sums[cur], reinterpret_cast<const float*>(S.pose[iT]),
-                                       reinterpret_cast<const float*>(S.plo[iT]),
+      if (warp == kRejectWarp && !first && !last) {
+        const bool stop = lm_candidate(S.sums[cur], reinterpret_cast<const float*>(S.pose[iT]), S.plo[iT],
                                        d.c.lambda_pow[min(k + 1, kLambdaPow) + kLambdaPow], d.c.eps_t2f, d.c.eps_r2f,
-                                       reinterpret_cast<float*>(S.pose[iR]), reinterpret_cast<float*>(S.plo[iR]), lane);
-        if (lane == 0) S.stop[1] = stop;
+                                       reinterpret_cast<float*>(S.pose[iR]), S.plo[iR], lane);
+        if (lane == 0) S.stop[eval & 1u][1] = stop;
       }
       __syncthreads();
-      if (!s_arrived) {
-        if (threadIdx.x == 0) atomicOr(d.status, ST_BARRIER);
-        failed = true;
-        break;
-      }
-      // every CTA of the group: FP32 reduction of the chunk partials in a fixed
-      // order (lane-strided sums, then a shuffle tree), one warp per word of
-      // three components; a word without this evaluation's tag is read again
-      // until it has it
-      bool ok = true;
+      // FP32 reduction of the chunk partials in a fixed order (lane-strided
+      // sums, then a shuffle tree), one warp per word of three components;
+      // words without this evaluation's tag are read again, all together,
+      // until they have it
+      bool ok = S.arrived != 0;
       float* sums = S.sums[cur ^ 1];
-      if (warp < kRegWords) {
+      if (warp < kRegWords && ok) {
         const ulonglong2* row = part + warp * d.max_slots;
-        // all loads are issued together (one L2 round trip), then checked and
-        // added in order
         constexpr int kLoads = (kRegChunks + 31) / 32;
         ulonglong2 w[kLoads];
 #pragma unroll
-        for (int u = 0; u < kLoads; ++u) {
-          const int q = lane + 32 * u;
-          w[u] = make_ulonglong2(0ull, 0ull);
-          if (q < nchunks) w[u] = ld_relaxed_gpu_b128(row + q);
+        for (int u = 0; u < kLoads; ++u) w[u] = make_ulonglong2(0ull, (unsigned long long)~tag << 32);
+        long long spins = 0;
+        for (;;) {
+          bool here = true;
+#pragma unroll
+          for (int u = 0; u < kLoads; ++u)
+            if (lane + 32 * u < nchunks && (unsigned)(w[u].y >> 32) != tag)
+              w[u] = ld_relaxed_gpu_b128(row + lane + 32 * u);
+#pragma unroll
+          for (int u = 0; u < kLoads; ++u)
+            here = here && (lane + 32 * u >= nchunks || (unsigned)(w[u].y >> 32) == tag);
+          if (__all_sync(0xffffffffu, here)) break;
+          if (++spins > d.spin_limit) {
+            ok = false;
+            break;
+          }
+          if (spins > 4096) __nanosleep(64);
         }
         float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
 #pragma unroll
         for (int u = 0; u < kLoads; ++u) {
-          const int q = lane + 32 * u;
-          if (q < nchunks) {
-            ok = ok && await_tag(row + q, w[u], tag, d.spin_limit);
+          if (lane + 32 * u < nchunks) {
             s0 += __uint_as_float((unsigned)w[u].x);
             s1 += __uint_as_float((unsigned)(w[u].x >> 32));
             s2 += __uint_as_float((unsigned)w[u].y);
@@ -774,15 +829,14 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
       if (warp == 0 && !last) {
         const int from = first ? iT : iC;
         const int ka = first ? 0 : max(k - 1, -kLambdaPow);
-        const bool stop = lm_candidate(sums, reinterpret_cast<const float*>(S.pose[from]),
-                                       reinterpret_cast<const float*>(S.plo[from]), d.c.lambda_pow[ka + kLambdaPow],
-                                       d.c.eps_t2f, d.c.eps_r2f, reinterpret_cast<float*>(S.pose[iA]),
-                                       reinterpret_cast<float*>(S.plo[iA]), lane);
-        if (lane == 0) S.stop[0] = stop;
+        const bool stop = lm_candidate(sums, reinterpret_cast<const float*>(S.pose[from]), S.plo[from],
+                                       d.c.lambda_pow[ka + kLambdaPow], d.c.eps_t2f, d.c.eps_r2f,
+                                       reinterpret_cast<float*>(S.pose[iA]), S.plo[iA], lane);
+        if (lane == 0) S.stop[eval & 1u][0] = stop;
       }
-      if (threadIdx.x == 32) {
+      if (warp == kDecideWarp && lane == 0) {
         const float En = sums[27];
-        const unsigned Nn = (unsigned)(sums[28] + 0.5f);  // below 2^24 as are the products' factors
+        const unsigned Nn = (unsigned)(sums[28] + 0.5f);  // below 2^24, as the comparison's factors must be
         const bool enough = (long long)Nn >= d.c.min_valid;
         const bool accept = first || (enough && prod_less(En, S.N, S.E, Nn));
         S.info.evals++;
@@ -790,62 +844,45 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
         if (accept) {
           S.E = En;
           S.N = Nn;
-          S.fin_E = En;
-          S.fin_N = Nn;
         }
         S.accept = accept ? (first && !enough ? 2 : 1) : 0;  // 2: too few pixels, the level ends
       }
       __syncthreads();
-      ++eval;
       // every thread follows the decision: slots and damping
       const int accept = S.accept;
+      const bool converged = accept != 2 && !last && S.stop[eval & 1u][accept ? 0 : 1] != 0;
       if (accept) {
         cur ^= 1;
-        if (first) {
-          k = 0;
-          const int t = iC;  // the candidate slot is free: the next candidate takes it
-          iC = iA;
-          iA = t;
-        } else {
-          k = max(k - 1, -kLambdaPow);
-          moved = true;
-          const int t = iT;
-          iT = iC;
-          iC = iA;
-          iA = t;
-        }
+        k = first ? 0 : max(k - 1, -kLambdaPow);
+        moved = moved || !first;
+        const int t = first ? iC : iT;  // the slot that is free now
+        if (!first) iT = iC;
+        iC = iA;
+        iA = t;
       } else {
         k = min(k + 1, kLambdaPow);
         const int t = iC;
         iC = iR;
         iR = t;
       }
-      if (accept == 2) {
-        done = true;
-      } else if (!last && S.stop[accept ? 0 : 1]) {
-        done = true;
-        if (threadIdx.x == 0) S.info.converged[l] = 1;
-      }
+      ++eval;
+      done = accept == 2 || converged;
+      if (converged && threadIdx.x == 0) S.info.converged[l] = 1;
     }
   }
   leave_registration(d, G, tag0);
-  if (failed) return;
-  if (lb == 0) {
-    if (threadIdx.x < 16) {  // the pose in FP64: hi + lo of each entry, the last row 0 0 0 1
-      const int q = threadIdx.x;
-      double t = q == 15 ? 1.0 : 0.0;
-      if (q < 12)
-        t = moved ? (double)reinterpret_cast<const float*>(S.pose[iT])[q] +
-                        (double)reinterpret_cast<const float*>(S.plo[iT])[q]
-                  : S.T0[q];
-      d.T_out[q] = t;
-    }
-    if (threadIdx.x == 0 && d.info) {
-      rf_track_info out = S.info;
-      out.final_cost = S.fin_N > 0u ? (double)S.fin_E / (double)S.fin_N : 0.0;
-      out.final_valid = (int64_t)S.fin_N;
-      *d.info = out;
-    }
+  if (failed || lb != 0) return;
+  if (threadIdx.x < 16) {  // the pose in FP64: hi + lo of each entry, the last row 0 0 0 1
+    const int q = threadIdx.x;
+    double t = q == 15 ? 1.0 : 0.0;
+    if (q < 12) t = moved ? (double)reinterpret_cast<const float*>(S.pose[iT])[q] + (double)S.plo[iT][q] : S.T0[q];
+    d.T_out[q] = t;
+  }
+  if (threadIdx.x == 0 && d.info) {
+    rf_track_info out = S.info;
+    out.final_cost = S.N > 0u ? (double)S.E / (double)S.N : 0.0;
+    out.final_valid = (int64_t)S.N;
+    *d.info = out;
   }
 }
 

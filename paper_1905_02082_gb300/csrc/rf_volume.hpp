@@ -52,7 +52,7 @@ struct rf_volume {
   rf::IntegState* d_integ = nullptr;
   int* d_tilemax = nullptr;
   uint16_t* d_dmask = nullptr;  // per pixel: raw depth if valid and not masked, else 0
-  int4* d_cand = nullptr;  // also the registration's pixel records (max_candidates or max_w * max_h entries, the larger)
+  int4* d_cand = nullptr;  // also the registration's pixel records (reg_records)
 
   // whole-frame staging (graph-replayed pipeline reads only these)
   uint16_t* d_depth = nullptr;
