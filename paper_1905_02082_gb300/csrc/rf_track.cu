@@ -29,6 +29,7 @@
 // A level ends early when the step falls below the thresholds.  Results are
 // deterministic: fixed chunks, fixed pixel-to-thread mapping, fixed reduction
 // order.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -60,6 +61,11 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
 __device__ __forceinline__ f2 mul2(f2 a, f2 b) {
   f2 r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ f2 sub2(f2 a, f2 b) {
@@ -114,15 +120,17 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
   const float py = fmaf(r1.z, z, fmaf(r1.y, y, r1.x * x)) + r1.w;
   const float pz = fmaf(r2.z, z, fmaf(r2.y, y, r2.x * x)) + r2.w;
   const float qx = px * c.inv_voxel, qy = py * c.inv_voxel, qz = pz * c.inv_voxel;
-  // block coordinates within +-kMaxCoord (a NaN fails too); |q| < 2^22 then
-  // makes the rounding trick below an exact floor
-  constexpr float kLo = -8.0f * kMaxCoord, kHi = 8.0f * kMaxCoord + 8.0f;
-  if (!(qx >= kLo && qy >= kLo && qz >= kLo && qx < kHi && qy < kHi && qz < kHi)) return kEmpty;
+  // floor: adding 1.5 * 2^23 rounded down leaves the integer in the low
+  // mantissa bits (exact for |q| < 2^22)
   const float tx = __fadd_rd(qx, kRound), ty = __fadd_rd(qy, kRound), tz = __fadd_rd(qz, kRound);
   const int kx = __float_as_int(tx) - 0x4B400000, ky = __float_as_int(ty) - 0x4B400000,
             kz = __float_as_int(tz) - 0x4B400000;
   const float fx = qx - (tx - kRound), fy = qy - (ty - kRound), fz = qz - (tz - kRound);
   const int bx = kx >> 3, by = ky >> 3, bz = kz >> 3;
+  // block coordinates from -kMaxCoord to kMaxCoord + 1 (no stored block has
+  // the latter); larger |q|, infinities and NaN give k beyond +-2^21 above
+  static_assert(kMaxCoord == 8191, "one comparison covers the three ranges");
+  if ((unsigned)((bx + kMaxCoord) | (by + kMaxCoord) | (bz + kMaxCoord)) >= 16384u) return kEmpty;
   // the cached entry's upper 42 bits are the block key (bx, by, bz: 14 bits each)
   const unsigned khi = ((unsigned)bx << 18) | (((unsigned)by & 0x3FFFu) << 4) | (((unsigned)bz >> 10) & 15u);
   const unsigned klo = (unsigned)bz << 22;
@@ -139,7 +147,7 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
   const int lx = kx & 7, ly = ky & 7, lz = kz & 7;
   int a0 = pool, a1 = pool, a2 = pool, a3 = pool;  // pools of the corners at dx = 0: (dy, dz) = 00, 10, 01, 11
   int b0 = pool, b1 = pool, b2 = pool, b3 = pool;  // and at dx = 1
-  if (lx == 7 || ly == 7 || lz == 7) {
+  if (((lx + 1) | (ly + 1) | (lz + 1)) & 8) {
     const int4 n0 = __ldg(v.nbr + 2 * (size_t)pool), n1 = __ldg(v.nbr + 2 * (size_t)pool + 1);
     const bool ex = lx == 7, ey = ly == 7, ez = lz == 7;
     const int m0 = ex ? n0.y : n0.x, m1 = ex ? n0.w : n0.z, m2 = ex ? n1.y : n1.x, m3 = ex ? n1.w : n1.z;
@@ -193,11 +201,12 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
       }
       colour = m != 255u;
     }
-    const f2 fx2 = pk(fx, fx);
+    const f2 fx2 = pk(fx, fx), unbias = pk(-0.0f, -kBias);
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-      d[n] = sub2(pk(F[2 * n + 1], I[2 * n + 1]), pk(F[2 * n], I[2 * n]));
-      e[n] = fma2(fx2, d[n], pk(F[2 * n], I[2 * n] - kBias));
+      const f2 p = pk(F[2 * n], I[2 * n]);
+      d[n] = sub2(pk(F[2 * n + 1], I[2 * n + 1]), p);
+      e[n] = fma2(fx2, d[n], add2(p, unbias));
     }
   }
   const f2 fy2 = pk(fy, fy), fz2 = pk(fz, fz);
@@ -217,7 +226,7 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
   gx = mul2(gx, gs);
   gy = mul2(gy, gs);
   gz = mul2(gz, gs);
-  const f2 r = fma2(val, pk(c.sdf_scale, colour ? c.col_scale : 0.0f), pk(0.0f, colour ? off : 0.0f));
+  const f2 r = pk(ST == RF_STORAGE_FP32 ? V : V * c.sdf_scale, colour ? fmaf(I, c.col_scale, off) : 0.0f);
   f2 J[6];
   J[0] = gx;
   J[1] = gy;
@@ -484,9 +493,9 @@ constexpr int kRegWarps = kRegThreads / 32;
 // depend on how many CTAs run the registration.  At most kRegChunks chunks
 // (one per CTA of a registration that has the GPU to itself, 98.7 % of the
 // SMs), of at least 128 pixels and a whole number of warps.
-__device__ __forceinline__ int chunk_pixels(int npix) {
-  const int c = (npix + kRegChunks - 1) / kRegChunks;
-  return max(128, (c + 127) & ~127);
+__host__ __device__ __forceinline__ int chunk_pixels(int npix) {
+  const int c = ((npix + kRegChunks - 1) / kRegChunks + 127) & ~127;
+  return c > 128 ? c : 128;
 }
 
 // Position in the frame of sample i of a level (row = i / Ws by a reciprocal
@@ -561,11 +570,16 @@ __device__ __forceinline__ void leave_registration(const RegDesc& d, int G, unsi
 // Exchange of the partial sums: evaluation e of the registration tags its
 // partials with base + e + 1 (base: d.tags[0]) and then counts the CTA in
 // d.tags[2] with a relaxed reduction; every CTA waits until the count shows
-// all G arrivals of e, then reads the partials, re-polling any word that does
-// not carry the tag yet (no fence orders a CTA's partials before its count,
-// so the tags carry the ordering).  The count also makes double buffering by
-// evaluation parity safe: a CTA writes evaluation e + 2 only after all G CTAs
-// arrived at e + 1, each after it had read all of evaluation e.
+// (nearly) all G arrivals of e, then reads the partials, re-polling any word
+// that does not carry the tag yet (no fence orders a CTA's partials before its
+// count, so the tags carry the ordering).  Where every CTA of a large group
+// has a chunk the last eighth of the arrivals is not waited for: the reads' round trip then
+// passes while the slowest CTAs finish (640x480 registration 108.7 -> 104.2
+// us, 1280x720 213.6 -> 206.1; with no count at all the polling readers slow
+// those CTAs down: 220.2).  Double buffering by evaluation parity is safe: a
+// CTA writes evaluation e + 2 only after it has read the words of e + 1 of
+// every CTA that has a chunk, and, where some CTA has none, after all G CTAs
+// arrived at e + 1; a CTA does either only after it has read all of e.
 //
 // Little of the LM step follows the reduction: while the CTA waits for the
 // others, one of its warps computes the next candidate of a rejection (it
@@ -674,6 +688,7 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
       const int i = bounds(lb + G * slot, end);
       if (i < end) fetch(i);
     }
+    const unsigned slack = G >= 64 && nchunks >= G && d.bar_extra == 0u ? (unsigned)G / 8u : 0u;
     bool done = false;
     int k = 0;  // damping lambda0 10^k: rejections minus acceptances
     for (int it = 0; it <= iters && !done; ++it) {
@@ -758,7 +773,7 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
       }
       if (lb >= nchunks && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
       if (threadIdx.x == 0)
-        S.arrived = await_count(d.tags + 2, (eval + 1u) * (unsigned)G + d.bar_extra, d.spin_limit);
+        S.arrived = await_count(d.tags + 2, (eval + 1u) * (unsigned)G + d.bar_extra - slack, d.spin_limit);
       // meanwhile: the next candidate should this one be rejected
       if (warp == kRejectWarp && !first && !last) {
         const bool stop = lm_candidate(S.sums[cur], reinterpret_cast<const float*>(S.pose[iT]), S.plo[iT],
@@ -975,7 +990,14 @@ rf_status launch_track(rf_volume* vol, const DevFrame& f, const double* T_init, 
   void* args[] = {&d};
   const void* fn = vol->p.storage == RF_STORAGE_FP16 ? (const void*)k_register<RF_STORAGE_FP16>
                                                      : (const void*)k_register<RF_STORAGE_FP32>;
-  return launch_coop(vol, fn, vol->reg_grid, args, st);
+  // no more CTAs than the finest level has chunks: then every CTA has pixels
+  // at every level of more than kRegChunks * 128 samples (see register_body)
+  int most = 1;
+  for (int l = 0; l < 3; ++l) {
+    const int s = vol->p.lm_strides[l], n = ((f.W + s - 1) / s) * ((f.H + s - 1) / s), c = chunk_pixels(n);
+    most = std::max(most, (n + c - 1) / c);
+  }
+  return launch_coop(vol, fn, std::min(vol->reg_grid, most), args, st);
 }
 
 rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const int* cta_stream, const int* first,
