@@ -183,9 +183,9 @@ rf_status rf_compute_mask(rf_volume* vol, const rf_frame* frame, const double* T
  * budget owns all device memory, or a frame loop with a latency bound that
  * cannot afford cudaMalloc's implicit device synchronisation.  The paper has
  * no counterpart; this is a property of the library only.
- *  - Allocates nothing: the per-call scratch (seed image, flood-fill working
- *    mask, barrier words, sweep flags) is one static device array of about
- *    1.9 MB that every GPU loading this library holds until the process exits.
+ *  - Allocates nothing: the per-call scratch (seed image, flood-fill
+ *    tiles, barrier words, sweep flags) is one static device array of about
+ *    0.9 MB that every GPU loading this library holds until the process exits.
  *  - Frames of at most 921,600 pixels (1280 x 720); larger frames return
  *    RF_ERR_INVALID_ARG with a message.  The flood fill is bounded by
  *    min(max_ff_sweeps, 4096) sweeps.

@@ -164,21 +164,22 @@ rf_status volume_buffers(rf_volume* vol, const rf_params* p, int64_t n_buckets, 
   const size_t max_slots = reg_slots(npix);
   const size_t ntiles = ((size_t)(max_width + kTile - 1) / kTile) * ((max_height + kTile - 1) / kTile);
   const size_t nslots = (size_t)n_buckets * kSlots;
+  const size_t fill_words = (size_t)kFillTileWords * ((max_width + 31) / 32) * ((max_height + 31) / 32);
   rf_status s;
   if ((s = A(&vol->d_hash, nslots, "hash")) || (s = A(&vol->d_vox, (size_t)max_blocks * kBV, "voxels")) ||
       (s = A(&vol->d_W, p->storage == RF_STORAGE_FP32 ? (size_t)max_blocks * kBV : 1, "weights")) ||
       (s = A(&vol->d_coords, (size_t)max_blocks, "coords")) ||
       (s = A(&vol->d_nbr, 2 * (size_t)max_blocks, "neighbour tables")) || (s = A(&vol->d_nblocks, 1, "pool")) ||
       (s = A(&vol->d_status, 1, "status")) || (s = A(&vol->d_regtags, 3, "registration tags")) ||
-      (s = A(&vol->d_partials, 2 * kRegWords * max_slots, "partials")) || (s = A(&vol->d_seeds, npix, "seeds")) ||
-      (s = A(&vol->d_md, npix, "mask work")) || (s = A(&vol->d_ff, (size_t)p->max_ff_sweeps + 2, "flood-fill words")) ||
+      (s = A(&vol->d_partials, 2 * kRegWords * max_slots, "partials")) ||
+      (s = A(&vol->d_tiles, fill_words, "flood-fill tiles")) || (s = A(&vol->d_ff, kFillWords, "mask words")) ||
       (s = A(&vol->d_integ, 1, "integ")) || (s = A(&vol->d_tilemax, ntiles, "tiles")) ||
       (s = A(&vol->d_dmask, npix, "masked depth")) ||
       // (a registration keeps its pixel records in the candidate list's memory:
       // the two never run at the same time on one volume)
       (s = A(&vol->d_cand, std::max((size_t)p->max_candidates, reg_records(p, max_width, max_height)), "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
       (s = A(&vol->d_rgb, npix * 3, "rgb staging")) || (s = A(&vol->d_mask, npix, "mask staging")) ||
-      (s = A(&vol->d_T, 48, "poses")) || (s = A(&vol->d_info, 1, "info")) || (s = A(&vol->d_guard, 1, "guard count")) ||
+      (s = A(&vol->d_T, 48, "poses")) || (s = A(&vol->d_info, 1, "info")) ||
       (s = A(&vol->d_pxcache, npix, "pixel block cache")))
     return s;
   return RF_OK;
@@ -379,9 +380,7 @@ struct BatchStage {
   double* T_out;
   uint8_t* mask_out;  // nullable
   uint8_t* mask_buf;  // the volume's mask (zeroed for a first frame: nothing is masked)
-  unsigned* guard;    // the volume's seed guard count and flood-fill words, zeroed
-  unsigned* ff;       // for a tracked frame
-  int ff_words;
+  unsigned* ff;       // the volume's mask words, zeroed for a tracked frame
   int npix;
   int mode;  // kModeTrack, kModeFirst or kModeIdle; the gate of the stream's kernels
 };
@@ -390,8 +389,8 @@ struct rf_batch_graph {
   std::vector<double> sig;  // per stream: H, W, fx, fy, cx, cy
   cudaGraphExec_t exec = nullptr;
   RegDesc* d_desc = nullptr;   // [2][n]: first and second registration
-  FloodDesc* d_flood = nullptr;  // [n]: the flood fills
-  MaskDesc* d_mask = nullptr;    // [n]: seeds, erosion, dilation
+  FillDesc* d_flood = nullptr;  // [n]: erosion, flood fill, dilation
+  MaskDesc* d_mask = nullptr;   // [n]: seeds
   // [n] BatchStage, then per registration launch (ngroups of them): CTA ->
   // stream [total], then the n + 1 group starts
   void* d_table = nullptr;
@@ -449,10 +448,7 @@ __global__ void __launch_bounds__(256) k_batch_stage(const BatchStage* __restric
     copy_bytes(b.rgb_dst, b.rgb_src, (size_t)b.npix * 3, tid, nth);
   }
   if (b.mode == kModeFirst) zero_bytes(b.mask_buf, (size_t)b.npix, tid, nth);
-  if (b.mode == kModeTrack && blockIdx.x == 0) {
-    for (int k = threadIdx.x; k < b.ff_words; k += blockDim.x) b.ff[k] = 0u;
-    if (threadIdx.x == 0) *b.guard = 0u;
-  }
+  if (b.mode == kModeTrack && blockIdx.x == 0 && threadIdx.x < kFillWords) b.ff[threadIdx.x] = 0u;
   if (blockIdx.x == 0 && threadIdx.x < 48) {
     const int k = threadIdx.x;
     if (k < 16 || b.mode != kModeTrack) b.T_dst[k] = b.T_src[k & 15];
@@ -527,17 +523,17 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     desc[i] = make_reg_desc(v, f[i], v->d_T, nullptr, v->d_T + 16, nullptr);
     desc[n + i] = make_reg_desc(v, f[i], v->d_T + 16, v->d_mask, v->d_T + 32, v->d_info);
   }
-  std::vector<FloodDesc> flood(n);
+  std::vector<FillDesc> flood(n);
   std::vector<MaskDesc> mdesc(n);
   for (int i = 0; i < n; ++i) {
     rf_volume* v = b->vols[i];
-    flood[i] = make_flood_desc(v, f[i]);
-    mdesc[i] = make_mask_desc(v, f[i], v->d_T + 16, v->d_mask);
+    flood[i] = make_fill_desc(v, f[i], v->d_mask);
+    mdesc[i] = make_mask_desc(v, f[i], v->d_T + 16);
   }
   e = cudaMalloc(&out->d_desc, sizeof(RegDesc) * desc.size());
   if (e == cudaSuccess) e = cudaMemcpy(out->d_desc, desc.data(), sizeof(RegDesc) * desc.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&out->d_flood, sizeof(FloodDesc) * n);
-  if (e == cudaSuccess) e = cudaMemcpy(out->d_flood, flood.data(), sizeof(FloodDesc) * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMalloc(&out->d_flood, sizeof(FillDesc) * n);
+  if (e == cudaSuccess) e = cudaMemcpy(out->d_flood, flood.data(), sizeof(FillDesc) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&out->d_mask, sizeof(MaskDesc) * n);
   if (e == cudaSuccess) e = cudaMemcpy(out->d_mask, mdesc.data(), sizeof(MaskDesc) * n, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return batch_error(b, RF_ERR_CUDA, std::string("batch descriptors: ") + cudaGetErrorString(e));
@@ -558,21 +554,23 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     const int map_len = out->total_ctas + n + 1;
     const int* ff_maps = maps + out->ngroups * map_len;
     const int ff_len = out->ff_ctas + n + 1;
-    int max_npix = 1;
-    for (int i = 0; i < n; ++i) max_npix = std::max(max_npix, f[i].H * f[i].W);
+    int max_npix = 1, max_seed_blocks = 1;
+    for (int i = 0; i < n; ++i) {
+      max_npix = std::max(max_npix, f[i].H * f[i].W);
+      max_seed_blocks = std::max(max_seed_blocks, mask_seed_blocks(f[i].H, f[i].W));
+    }
     const dim3 copy_grid((unsigned)std::min((max_npix * 3 / 16 + 255) / 256, 64), (unsigned)n);
     k_batch_stage<<<copy_grid, 256, 0, cs>>>(table);
     for (int gi = 0; gi < out->ngroups && !s; ++gi)
       s = launch_register_batch(b->vols[0], out->d_desc, maps + gi * map_len, maps + gi * map_len + out->total_ctas,
                                 out->total_ctas, cs);
-    // residual seeds and erosion of every stream: one launch each (guard
-    // counts and flood-fill words were reset by the staging kernel); flood
-    // fills: one cooperative launch per group of streams; dilation: one launch
-    if (!s) s = launch_mask_pre_batch(b->vols[0], out->d_mask, n, max_npix, cs);
+    // residual seeds of every stream: one launch (the mask words were reset by
+    // the staging kernel); erosion, flood fill and dilation: one cooperative
+    // launch per group of streams
+    if (!s) s = launch_seeds_batch(b->vols[0], out->d_mask, n, max_seed_blocks, cs);
     for (int gi = 0; gi < out->ngroups && !s; ++gi)
-      s = launch_floodfill_batch(b->vols[0], out->d_flood, ff_maps + gi * ff_len,
-                                 ff_maps + gi * ff_len + out->ff_ctas, out->ff_ctas, cs);
-    if (!s) s = launch_mask_post_batch(b->vols[0], out->d_mask, n, max_npix, cs);
+      s = launch_fill_batch(b->vols[0], out->d_flood, ff_maps + gi * ff_len, ff_maps + gi * ff_len + out->ff_ctas,
+                            out->ff_ctas, cs);
     for (int gi = 0; gi < out->ngroups && !s; ++gi)
       s = launch_register_batch(b->vols[0], out->d_desc + n, maps + gi * map_len,
                                 maps + gi * map_len + out->total_ctas, out->total_ctas, cs);
@@ -658,9 +656,9 @@ rf_status rf_destroy_volume(rf_volume* vol) {
   for (auto& e : vol->ev)
     if (e) cudaEventDestroy(e);
   void* dev[] = {vol->d_hash, vol->d_vox,  vol->d_W,       vol->d_coords, vol->d_nbr, vol->d_nblocks, vol->d_status,
-                 vol->d_regtags, vol->d_partials, vol->d_seeds, vol->d_md,    vol->d_ff,      vol->d_integ,
+                 vol->d_regtags, vol->d_partials, vol->d_tiles, vol->d_ff,      vol->d_integ,
                  vol->d_tilemax, vol->d_cand, vol->d_depth, vol->d_rgb,   vol->d_mask,    vol->d_T, vol->d_info,
-                 vol->d_guard, vol->d_pxcache, vol->d_dmask};
+                 vol->d_pxcache, vol->d_dmask};
   for (void* p : dev)
     if (p) cudaFree(p);
   delete vol;
@@ -703,6 +701,7 @@ rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_bl
     rf_destroy_volume(vol);
     return s;
   }
+  vol->d_guard = vol->d_ff;
   vol->dv.hash = vol->d_hash;
   vol->dv.bucket_mask = (unsigned long long)n_buckets - 1;
   vol->dv.vox = vol->d_vox;
@@ -1232,9 +1231,7 @@ rf_status rf_batch_process(rf_batch* b, const rf_frame* frames, const double* co
     t.T_out = T_out_dev[i];
     t.mask_out = mask_dev ? mask_dev[i] : nullptr;
     t.mask_buf = v->d_mask;
-    t.guard = v->d_guard;
     t.ff = v->d_ff;
-    t.ff_words = 2 + v->p.max_ff_sweeps;
     t.npix = frames[i].height * frames[i].width;
     t.mode = mode[i];
     if (mode[i] == kModeTrack) tracked.push_back(i);

@@ -166,16 +166,14 @@ struct IntegState {
   float szf[3];
 };
 
-// Everything one stream's residual seeds, erosion and dilation need.
+// Everything one stream's residual seeds need.
 struct MaskDesc {
   DevVol v;
   DevFrame f;
   DevParams p;
   const double* T;  // first-registration pose
-  uint8_t* seeds;
+  unsigned* tiles;  // as FillDesc's
   unsigned* guard;
-  uint8_t* md;
-  uint8_t* mask_out;
   const unsigned long long* pxcache;  // the volume's per-pixel block cache (read only)
 };
 
@@ -369,18 +367,21 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, un
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* vgen = bar + 1;
-    const unsigned gen = *vgen;
-    __threadfence();
-    const unsigned ticket = atomicAdd(bar, 1u);
+    // release and acquire on the accesses themselves (with the CTA barriers
+    // they order every thread's accesses); separate fences around them tripled
+    // the barrier's time
+    unsigned gen, ticket, now;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(gen) : "l"(bar + 1) : "memory");
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(ticket) : "l"(bar) : "memory");
     int ok = 1;
     if (ticket == nblocks + extra - 1) {
-      atomicExch(bar, 0u);
-      __threadfence();
-      atomicAdd(bar + 1, 1u);
+      asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
     } else {
       long long spins = 0;
-      while (*vgen == gen) {
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar + 1) : "memory");
+        if (now != gen) break;
         if (++spins > spin_limit) {
           ok = 0;
           atomicOr(status, ST_BARRIER);
@@ -389,7 +390,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, un
         if (spins > 4096) __nanosleep(64);  // spin first: most waits are short
       }
     }
-    __threadfence();
     s_ok = ok;
   }
   __syncthreads();
@@ -471,12 +471,11 @@ rf_status launch_mask(rf_volume* vol, const DevFrame& f, const double* T, uint8_
 rf_status launch_virtual_depth(rf_volume* vol, const DevFrame& f, const double* T, unsigned far_raw, uint16_t* out,
                                cudaStream_t st);
 rf_status launch_integrate(rf_volume* vol, const DevFrame& f, const double* T, const uint8_t* mask, cudaStream_t st);
-// residual seeds + erosion, and dilation, of several streams in one launch
-// each (grid y = stream; max_npix bounds every stream's pixel count; the
-// guard counts and flood-fill words are reset by the caller)
-MaskDesc make_mask_desc(rf_volume* vol, const DevFrame& f, const double* T, uint8_t* mask_out);
-rf_status launch_mask_pre_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_npix, cudaStream_t st);
-rf_status launch_mask_post_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_npix, cudaStream_t st);
+// residual seeds of several streams in one launch (grid y = stream; max_blocks:
+// the largest mask_seed_blocks; the mask words are reset by the caller)
+int mask_seed_blocks(int H, int W);
+MaskDesc make_mask_desc(rf_volume* vol, const DevFrame& f, const double* T);
+rf_status launch_seeds_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_blocks, cudaStream_t st);
 // profiling events (no-ops unless profiling is enabled); ids below
 enum ProfEvent { EV_FRAME0, EV_TRACK1_END, EV_MASK_END, EV_TRACK2_END, EV_INTEG0, EV_KERNEL0, EV_KERNEL1, EV_FRAME1,
                  EV_COUNT };
@@ -486,26 +485,23 @@ RegDesc make_reg_desc(rf_volume* vol, const DevFrame& f, const double* T_init, c
                       rf_track_info* info);
 rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const int* cta_stream, const int* first,
                                 int total_ctas, cudaStream_t st);
-// the three parts of launch_mask (the flood fill is the cooperative one)
-rf_status launch_mask_pre(rf_volume* vol, const DevFrame& f, const double* T, cudaStream_t st);
-rf_status launch_mask_ff(rf_volume* vol, const DevFrame& f, cudaStream_t st);
-// flood fills of several streams in one cooperative launch (the batches'
-// CTA maps; total_ctas must not exceed floodfill_max_grid)
-struct FloodDesc {
-  uint8_t* md;
-  const uint16_t* depth;
+// erosion, flood fill and dilation of several streams in one cooperative
+// launch (the batches' CTA maps; total_ctas must not exceed floodfill_max_grid)
+constexpr int kFillTileWords = 6 * 32 + 4;  // global memory of one 32 x 32 tile
+constexpr int kFillWords = 8;  // guard count, barrier (2), change flags (3), M_R not empty; zeroed per mask
+struct FillDesc {
+  uint8_t* mask_out;
+  unsigned* tiles;  // kFillTileWords per tile, written by the seeds
   int H, W;
-  long long theta_ppm;
   unsigned* ff;
   int max_sweeps;
   unsigned* status;
   long long spin_limit;
   unsigned bar_extra;
 };
-FloodDesc make_flood_desc(rf_volume* vol, const DevFrame& f);
-rf_status launch_floodfill_batch(rf_volume* vol, const FloodDesc* descs, const int* cta_stream, const int* first,
-                                 int total_ctas, cudaStream_t st);
-rf_status launch_mask_post(rf_volume* vol, const DevFrame& f, uint8_t* mask_out, cudaStream_t st);
+FillDesc make_fill_desc(rf_volume* vol, const DevFrame& f, uint8_t* mask_out);
+rf_status launch_fill_batch(rf_volume* vol, const FillDesc* descs, const int* cta_stream, const int* first,
+                            int total_ctas, cudaStream_t st);
 // neighbour tables of the blocks allocated since *lo_ptr (or since lo when lo_ptr is null)
 rf_status launch_nbr_fixup(rf_volume* vol, const int* lo_ptr, int lo, cudaStream_t st, const int* gate = nullptr);
 }  // namespace rf

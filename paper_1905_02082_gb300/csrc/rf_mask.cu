@@ -1,21 +1,21 @@
 // Dynamics detection (ReFusion Sec. III-C) on sm_103a.
 //
 //   k_seeds      r_i = V_SDF(T x_i)^2 (the residual of Eq. 2, V_SDF truncated to
-//                [-tau, tau]) and the raw mask r_i > t = gamma tau^2 (Eq. 5), one
-//                thread per pixel.  The
+//                [-tau, tau]) and the raw mask r_i > t = gamma tau^2 (Eq. 5), a
+//                warp per 32 pixels of a row, written as bits.  The
 //                decision is exact: the FP32 evaluation carries an error bound;
 //                when the lattice cell or the comparison is within it, the pixel
 //                is re-evaluated in FP64 with a fixed operation order and no
-//                contraction (__d*_rn), the order the FP64 oracle uses.
-//   k_erode      M_R = 3x3 erosion of the raw mask (outside the image = 0), and
-//                M_D initialised to M_R.
-//   k_floodfill  Alg. 1 closure: n joins from p when |D(p) - D(n)| < theta D(p)
-//                (4-neighbours, raw integer depth, theta in ppm).  The closure
-//                is the set reachable from M_R, independent of visiting order,
-//                so tiles propagate locally in shared memory until stable and
-//                sweep globally (cooperative launch, bounded grid barrier) until
-//                no tile changes; at most max_ff_sweeps sweeps.
-//   k_dilate     final mask = 3x3 dilation of M_D.
+//                contraction (__d*_rn), the order the FP64 oracle uses.  The
+//                warps also write the pixels' join conditions of Alg. 1, as bits.
+//   k_mask_fill  the rest, in one cooperative launch: M_R = 3x3 erosion of the raw
+//                mask (outside the image = 0); the closure of Alg. 1, in which n
+//                joins from p when |D(p) - D(n)| < theta D(p) (4-neighbours, raw
+//                integer depth, theta in ppm); the final mask = 3x3 dilation of
+//                M_D.  The closure is the set reachable from M_R, independent of
+//                visiting order, so it is taken tile by tile until nothing changes:
+//                at most max_ff_sweeps sweeps over the image, a grid-wide barrier
+//                (bounded) after each.
 #include <cmath>
 #include <mutex>
 
@@ -108,31 +108,48 @@ __device__ __forceinline__ int seed_fp32(const DevVol& v, const DevFrame& f, con
   return r > t ? 1 : 0;
 }
 
-// Seeds of the kSeedThreads * kSeedPx pixels of CTA `block` (blockDim.x =
-// kSeedThreads; pixel block * kSeedThreads * kSeedPx + j * kSeedThreads + tid
-// for j < kSeedPx).  Every thread first loads its pixels' depths and cache
-// entries, then decides them in FP32; the ambiguous ones are queued in shared
+__device__ __forceinline__ bool may_join(unsigned from, unsigned to, long long theta_ppm) {
+  const unsigned diff = from > to ? from - to : to - from;
+  return (long long)((unsigned long long)diff * 1000000u) < theta_ppm * (long long)from;
+}
+
+// Words of one tile of 32 x 32 pixels, row r of each plane at word 32 plane +
+// r: raw mask, joins from the left, from the right (bits reversed), from
+// above and from below, the flood fill's set M; then M's border: top row,
+// bottom row, left column, right column.
+constexpr int kSeedsPlane = 0, kRightPlane = 32, kLeftPlane = 64, kDownPlane = 96, kUpPlane = 128, kMPlane = 160,
+              kBorder = 192;
+static_assert(kBorder + 4 == kFillTileWords, "tile layout");
+
+// Seeds and join conditions of the kSeedThreads / 32 * kSeedPx row words (32
+// pixels of a row, the first one's column a multiple of 32) of CTA `block`.
+// Every thread first loads its pixels' depths and cache entries, then decides
+// them in FP32; the ambiguous ones are queued in shared
 // memory and decided in FP64 afterwards, side by side by consecutive threads:
 // on GB300 the FP64 pipe is narrow, and a warp that takes the FP64 branch for
 // one of its lanes costs as much as one that takes it for all 32.
-// pxcache: the registration's per-pixel block cache (nullptr: none), read
-// only, to skip hash probes.
+// The join conditions of Alg. 1 are decided here, where every SM has pixels and
+// the issue slots are idle (the lookups' latency bounds the kernel), and not in
+// the flood fill, which runs on few SMs (there they took 13 us of 640x480).
+// pxcache: the registration's per-pixel block cache, read only, to skip hash
+// probes.
 constexpr int kSeedThreads = 256;
 constexpr int kSeedPx = 4;
+constexpr int kSeedWords = kSeedThreads / 32 * kSeedPx;
 
-__host__ __device__ constexpr int seed_blocks(int npix) {
-  return (npix + kSeedThreads * kSeedPx - 1) / (kSeedThreads * kSeedPx);
-}
+__host__ __device__ constexpr int row_words(int W) { return (W + 31) / 32; }
+__host__ __device__ constexpr int seed_blocks(int H, int W) { return (H * row_words(W) + kSeedWords - 1) / kSeedWords; }
 
 template <int ST>
 __device__ __forceinline__ void seeds_body(const DevVol& v, const DevFrame& f, const DevParams& p,
-                                           const double* __restrict__ T, uint8_t* __restrict__ seeds,
+                                           const double* __restrict__ T, unsigned* __restrict__ tiles,
                                            unsigned* guard_count, const unsigned long long* __restrict__ pxcache,
                                            int block) {
   // pose and threshold converted once per CTA (conversions use the FP64 pipe)
   __shared__ float sR[12];
   __shared__ double s_t64;
-  __shared__ int s_queue[kSeedThreads * kSeedPx];
+  __shared__ unsigned short s_queue[kSeedWords * 32];
+  __shared__ unsigned s_words[kSeedWords];
   __shared__ int s_n;
   if (threadIdx.x < 12) {
     const int i = threadIdx.x < 9 ? threadIdx.x / 3 : threadIdx.x - 9;
@@ -142,283 +159,363 @@ __device__ __forceinline__ void seeds_body(const DevVol& v, const DevFrame& f, c
   if (threadIdx.x == 12) s_t64 = __dmul_rn(__dmul_rn(p.gamma_d, p.tau_d), p.tau_d);
   if (threadIdx.x == 13) s_n = 0;
   __syncthreads();
-  const int npix = f.H * f.W;
-  const int first = block * kSeedThreads * kSeedPx + (int)threadIdx.x;
-  unsigned raw[kSeedPx];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rw = row_words(f.W), nwords = f.H * rw;
+  auto word_of = [&](int local) { return block * kSeedWords + local; };  // local: 0 .. kSeedWords - 1
+  auto tile_word = [&](int w) {  // the place of row word w in its tile's planes
+    const int row = w / rw;
+    return tiles + (size_t)((row >> 5) * rw + (w - row * rw)) * kFillTileWords + (row & 31);
+  };
+  unsigned raw[kSeedPx], above[kSeedPx], below[kSeedPx], side[kSeedPx];
   unsigned long long cached[kSeedPx];
+  int us[kSeedPx], vs[kSeedPx];
 #pragma unroll
   for (int j = 0; j < kSeedPx; ++j) {
-    const int idx = first + j * kSeedThreads;
-    raw[j] = idx < npix ? __ldg(f.depth + idx) : 0u;
-    cached[j] = idx < npix && pxcache ? __ldg(pxcache + idx) : kEmpty;
+    const int w = word_of(j * (kSeedThreads / 32) + warp), row = w / rw;
+    const int u = (w - row * rw) * 32 + lane, idx = row * f.W + u;
+    const bool in = w < nwords && u < f.W;
+    us[j] = u;
+    vs[j] = row;
+    raw[j] = in ? __ldg(f.depth + idx) : 0u;
+    cached[j] = in ? __ldg(pxcache + idx) : kEmpty;
+    above[j] = in && row > 0 ? __ldg(f.depth + idx - f.W) : 0u;
+    below[j] = in && row + 1 < f.H ? __ldg(f.depth + idx + f.W) : 0u;
+    side[j] = in && lane == 0 && u > 0 ? __ldg(f.depth + idx - 1)
+              : in && lane == 31 && u + 1 < f.W ? __ldg(f.depth + idx + 1)
+                                                : 0u;
   }
 #pragma unroll 1
   for (int j = 0; j < kSeedPx; ++j) {
-    const int idx = first + j * kSeedThreads;
-    if (idx >= npix) break;
+    const int local = j * (kSeedThreads / 32) + warp, w = word_of(local);
+    if (w >= nwords) break;
     const unsigned rj = j == 0 ? raw[0] : (j == 1 ? raw[1] : (j == 2 ? raw[2] : raw[3]));
+    const unsigned aj = j == 0 ? above[0] : (j == 1 ? above[1] : (j == 2 ? above[2] : above[3]));
+    const unsigned bj = j == 0 ? below[0] : (j == 1 ? below[1] : (j == 2 ? below[2] : below[3]));
+    const unsigned sj = j == 0 ? side[0] : (j == 1 ? side[1] : (j == 2 ? side[2] : side[3]));
     const unsigned long long cj = j == 0 ? cached[0] : (j == 1 ? cached[1] : (j == 2 ? cached[2] : cached[3]));
+    const int u = j == 0 ? us[0] : (j == 1 ? us[1] : (j == 2 ? us[2] : us[3]));
+    const int vv = j == 0 ? vs[0] : (j == 1 ? vs[1] : (j == 2 ? vs[2] : vs[3]));
     int seed = 0;
-    if (pixel_valid(p, rj)) seed = seed_fp32<ST>(v, f, p, sR, idx % f.W, idx / f.W, rj, cj);
-    if (seed == 2) s_queue[atomicAdd(&s_n, 1)] = idx;
-    else seeds[idx] = (uint8_t)seed;
+    if (pixel_valid(p, rj)) seed = seed_fp32<ST>(v, f, p, sR, u, vv, rj, cj);  // (raw is 0 outside the image)
+    if (seed == 2) s_queue[atomicAdd(&s_n, 1)] = (unsigned short)(local * 32 + lane);
+    __syncwarp();
+    const unsigned seeds = __ballot_sync(0xffffffffu, seed == 1);
+    // join conditions (a depth of 0, also outside the image, joins nothing)
+    const unsigned dl = __shfl_up_sync(0xffffffffu, rj, 1), dr = __shfl_down_sync(0xffffffffu, rj, 1);
+    const unsigned jr = __ballot_sync(0xffffffffu, may_join(lane == 0 ? sj : dl, rj, p.theta_ppm));
+    const unsigned jl = __ballot_sync(0xffffffffu, may_join(lane == 31 ? sj : dr, rj, p.theta_ppm));
+    const unsigned jd = __ballot_sync(0xffffffffu, may_join(aj, rj, p.theta_ppm));
+    const unsigned ju = __ballot_sync(0xffffffffu, may_join(bj, rj, p.theta_ppm));
+    if (lane == 0) s_words[local] = seeds;
+    if (lane < 4) {
+      const unsigned x = lane == 0 ? jr : (lane == 1 ? __brev(jl) : (lane == 2 ? jd : ju));
+      tile_word(w)[kRightPlane + 32 * lane] = x;
+    }
   }
   __syncthreads();
   const int n = s_n;
   for (int i = threadIdx.x; i < n; i += kSeedThreads) {
-    const int idx = s_queue[i];
-    const double r64 = residual_fp64<ST>(v, f, p, T, idx % f.W, idx / f.W, __ldg(f.depth + idx));
-    seeds[idx] = (r64 >= 0.0 && r64 > s_t64) ? 1 : 0;
+    const int local = s_queue[i] >> 5, bit = s_queue[i] & 31, w = word_of(local), row = w / rw;
+    const int u = (w - row * rw) * 32 + bit;
+    const double r64 = residual_fp64<ST>(v, f, p, T, u, row, __ldg(f.depth + row * f.W + u));
+    if (r64 >= 0.0 && r64 > s_t64) atomicOr(&s_words[local], 1u << bit);
   }
   if (threadIdx.x == 0 && n > 0 && guard_count) atomicAdd(guard_count, (unsigned)n);
+  __syncthreads();
+  if (threadIdx.x < kSeedWords && word_of(threadIdx.x) < nwords)
+    tile_word(word_of(threadIdx.x))[kSeedsPlane] = s_words[threadIdx.x];
 }
 
 template <int ST>
 __global__ void __launch_bounds__(kSeedThreads) k_seeds(DevVol v, DevFrame f, DevParams p,
-                                                        const double* __restrict__ T, uint8_t* __restrict__ seeds,
+                                                        const double* __restrict__ T, unsigned* __restrict__ tiles,
                                                         unsigned* guard_count,
                                                         const unsigned long long* __restrict__ pxcache) {
-  if (gated_off(f.gate, kModeTrack)) return;
-  seeds_body<ST>(v, f, p, T, seeds, guard_count, pxcache, blockIdx.x);
+  seeds_body<ST>(v, f, p, T, tiles, guard_count, pxcache, blockIdx.x);
 }
 
 // grid (x, n streams): the seeds of every tracked stream of a batch.
 template <int ST>
 __global__ void __launch_bounds__(kSeedThreads) k_seeds_batch(const MaskDesc* __restrict__ descs) {
   const MaskDesc& d = descs[blockIdx.y];
-  if (gated_off(d.f.gate, kModeTrack) || (int)blockIdx.x >= seed_blocks(d.f.H * d.f.W)) return;
-  seeds_body<ST>(d.v, d.f, d.p, d.T, d.seeds, d.guard, d.pxcache, blockIdx.x);
+  if (gated_off(d.f.gate, kModeTrack) || (int)blockIdx.x >= seed_blocks(d.f.H, d.f.W)) return;
+  seeds_body<ST>(d.v, d.f, d.p, d.T, d.tiles, d.guard, d.pxcache, blockIdx.x);
 }
 
-__device__ __forceinline__ void erode_px(const uint8_t* __restrict__ in, int H, int W, uint8_t* __restrict__ mr,
-                                         int idx) {
-  const int u = idx % W, v = idx / W;
-  uint8_t all = 1;
-  if (u == 0 || v == 0 || u == W - 1 || v == H - 1) {
-    all = 0;
-  } else {
+// ---------------------------------------------------------------------------
+// Erosion, flood fill and dilation.  A warp holds a tile of 32 x 32 pixels as
+// bits, row r on lane r: the set M and four planes of join conditions (bit c
+// of row r: the pixel may join from its left / right / upper / lower
+// neighbour).  Within the tile a row fills to either side with one addition
+// (the carry runs through the joinable pixels) and the columns in five shuffle
+// steps each way, so a tile settles in a few hundred cycles, where a pixel per
+// thread and step took up to 512 CTA barriers.  The 4 x 4 tiles of a CTA
+// exchange their border rows and columns through shared memory until none
+// changes, then CTAs exchange theirs through global memory, a grid barrier per
+// sweep: an object of a few hundred pixels takes three or four sweeps.  Bound
+// by latency: barriers, and the chain of tiles an object extends over.
+// 640x480 with a moving object: erosion, fill and dilation 50 us before (three
+// kernels, 600 tiles of 32 x 16 in ~12 sweeps).
+// ---------------------------------------------------------------------------
+constexpr int kFillTx = 4, kFillTy = 4;  // tiles of a CTA's region
+constexpr int kFillThreads = 32 * kFillTx * kFillTy;
+// One tile in a warp's registers.
+struct Tile {
+  unsigned m;               // M
+  unsigned right, left_r;   // joins from the left neighbour, and (bits reversed) from the right one
+  unsigned down, up;        // joins from above and from below
+};
+
+// Bits of the row words that a fill towards higher bits reaches: `p` marks the
+// pixels that may join from the next lower bit.  Adding the first joining
+// pixels to p clears the run of ones above each of them.
+__device__ __forceinline__ unsigned fill_up_bits(unsigned m, unsigned p) {
+  const unsigned s = p & (m << 1), sum = p + s;
+  return m | s | (p & ~sum);
+}
+
+// Closure within the tile.
+__device__ __forceinline__ unsigned settle(Tile t, int lane) {
+  unsigned pd[5], pu[5];  // rows 1, 2, 4, 8, 16 above / below reach this one
+  pd[0] = lane == 0 ? 0u : t.down;
+  pu[0] = lane == 31 ? 0u : t.up;
 #pragma unroll
-    for (int dv = -1; dv <= 1; ++dv)
+  for (int k = 0; k < 4; ++k) {  // (a lane without a row that far away gets its own value: 0 there)
+    pd[k + 1] = pd[k] & __shfl_up_sync(0xffffffffu, pd[k], 1 << k);
+    pu[k + 1] = pu[k] & __shfl_down_sync(0xffffffffu, pu[k], 1 << k);
+  }
+  unsigned m = t.m, old;
+  do {
+    old = m;
+    m = fill_up_bits(m, t.right);
+    m = __brev(fill_up_bits(__brev(m), t.left_r));
 #pragma unroll
-      for (int du = -1; du <= 1; ++du) all &= (__ldg(in + (v + dv) * W + (u + du)) != 0);
+    for (int k = 0; k < 5; ++k) m |= pd[k] & __shfl_up_sync(0xffffffffu, m, 1 << k);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) m |= pu[k] & __shfl_down_sync(0xffffffffu, m, 1 << k);
+  } while (__any_sync(0xffffffffu, m != old));  // at most 1,024 times: each adds a pixel
+  return m;
+}
+
+// M_R, the 3x3 erosion of the raw mask, of tile (tx, ty); zero outside the
+// image.  All words are loaded before any is used.
+__device__ __forceinline__ unsigned erode_tile(const unsigned* __restrict__ tiles, int tiles_x, int H, int tx, int ty,
+                                               int lane) {
+  // row words of the tile and its left and right neighbour, of row y of the image
+  auto word = [&](int x, int y) {
+    return x >= 0 && x < tiles_x && y >= 0 && y < H
+               ? __ldcg(tiles + (size_t)((y >> 5) * tiles_x + x) * kFillTileWords + kSeedsPlane + (y & 31))
+               : 0u;
+  };
+  const int y = ty * 32 + lane, ya = ty * 32 - 1, yb = ty * 32 + 32;
+  const unsigned w = word(tx, y), l = word(tx - 1, y), r = word(tx + 1, y);
+  const unsigned aw = word(tx, ya), al = word(tx - 1, ya), ar = word(tx + 1, ya);
+  const unsigned bw = word(tx, yb), bl = word(tx - 1, yb), br = word(tx + 1, yb);
+  auto narrow = [](unsigned c, unsigned left, unsigned right) {
+    return c & ((c << 1) | (left >> 31)) & ((c >> 1) | (right << 31));
+  };
+  const unsigned h = narrow(w, l, r), above = narrow(aw, al, ar), below = narrow(bw, bl, br);
+  const unsigned hu = __shfl_up_sync(0xffffffffu, h, 1), hd = __shfl_down_sync(0xffffffffu, h, 1);
+  return h & (lane == 0 ? above : hu) & (lane == 31 ? below : hd);
+}
+
+// Border of M: top row, bottom row, left column, right column (on every lane).
+__device__ __forceinline__ uint4 border_of(unsigned m) {
+  return make_uint4(__shfl_sync(0xffffffffu, m, 0), __shfl_sync(0xffffffffu, m, 31),
+                    __ballot_sync(0xffffffffu, m & 1u), __ballot_sync(0xffffffffu, m >> 31));
+}
+
+// ff words: [1] barrier count, [2] barrier generation, [3 + s % 3] changed in
+// sweep s, [6] M_R is not empty (all zero at the start; [0] is the seeds' guard
+// count).  Run by a group of G CTAs, this one being number lb of the group.
+__device__ void mask_fill_body(const FillDesc& d, int lb, int G) {
+  __shared__ uint4 sb[2][kFillTx * kFillTy];  // the tiles' borders, by parity of the exchange
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wx = warp % kFillTx, wy = warp / kFillTx;
+  const int H = d.H, W = d.W;
+  const int tiles_x = (W + 31) / 32, tiles_y = (H + 31) / 32;
+  const int regs_x = (tiles_x + kFillTx - 1) / kFillTx;
+  const int nreg = regs_x * ((tiles_y + kFillTy - 1) / kFillTy);
+  const bool resident = nreg <= G;  // one region per CTA: its tiles stay in registers
+  volatile unsigned* changed = d.ff + 3;
+  auto tile_at = [&](int tx, int ty) -> int {
+    return tx >= 0 && ty >= 0 && tx < tiles_x && ty < tiles_y ? ty * tiles_x + tx : -1;
+  };
+  auto words = [&](int tile) { return d.tiles + (size_t)tile * kFillTileWords; };
+  auto border_word = [&](int tile, int k) { return tile >= 0 ? __ldcg(words(tile) + kBorder + k) : 0u; };
+  auto put_border = [&](int tile, const uint4& b) {
+    if (lane < 4) __stcg(words(tile) + kBorder + lane, lane == 0 ? b.x : (lane == 1 ? b.y : (lane == 2 ? b.z : b.w)));
+  };
+  auto load_planes = [&](int tile, int ty, Tile& x) {
+    const unsigned* w = words(tile) + lane;
+    const bool in = ty * 32 + lane < H;  // (rows below the image were not written)
+    x.right = in ? __ldcg(w + kRightPlane) : 0u;
+    x.left_r = in ? __ldcg(w + kLeftPlane) : 0u;
+    x.down = in ? __ldcg(w + kDownPlane) : 0u;
+    x.up = in ? __ldcg(w + kUpPlane) : 0u;
+  };
+  Tile t = {0u, 0u, 0u, 0u, 0u};
+  bool some = false;
+  for (int reg = lb; reg < nreg; reg += G) {
+    const int tx = reg % regs_x * kFillTx + wx, ty = reg / regs_x * kFillTy + wy, tile = tile_at(tx, ty);
+    if (tile < 0) continue;
+    t.m = erode_tile(d.tiles, tiles_x, H, tx, ty, lane);
+    some = some || t.m != 0u;
+    put_border(tile, border_of(t.m));
+    if (resident) load_planes(tile, ty, t);
+    else __stcg(words(tile) + kMPlane + lane, t.m);
   }
-  mr[idx] = all;
-}
-
-__global__ void __launch_bounds__(256) k_erode(const uint8_t* __restrict__ in, int H, int W, uint8_t* __restrict__ mr,
-                                               const int* gate) {
-  if (gated_off(gate, kModeTrack)) return;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < H * W) erode_px(in, H, W, mr, idx);
-}
-
-__device__ __forceinline__ void dilate_px(const uint8_t* __restrict__ in, int H, int W, uint8_t* __restrict__ out,
-                                          int idx) {
-  const int u = idx % W, v = idx / W;
-  uint8_t any = 0;
-  for (int dv = -1; dv <= 1; ++dv) {
-    const int y = v + dv;
-    if (y < 0 || y >= H) continue;
-    for (int du = -1; du <= 1; ++du) {
-      const int x = u + du;
-      if (x < 0 || x >= W) continue;
-      any |= (__ldg(in + y * W + x) != 0);
-    }
-  }
-  out[idx] = any;
-}
-
-__global__ void __launch_bounds__(256) k_dilate(const uint8_t* __restrict__ in, int H, int W, uint8_t* __restrict__ out,
-                                                const int* gate) {
-  if (gated_off(gate, kModeTrack)) return;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < H * W) dilate_px(in, H, W, out, idx);
-}
-
-// grid (x, n streams): erosion and dilation of every tracked stream of a batch.
-__global__ void __launch_bounds__(256) k_erode_batch(const MaskDesc* __restrict__ descs) {
-  const MaskDesc& d = descs[blockIdx.y];
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (gated_off(d.f.gate, kModeTrack) || idx >= d.f.H * d.f.W) return;
-  erode_px(d.seeds, d.f.H, d.f.W, d.md, idx);
-}
-
-__global__ void __launch_bounds__(256) k_dilate_batch(const MaskDesc* __restrict__ descs) {
-  const MaskDesc& d = descs[blockIdx.y];
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (gated_off(d.f.gate, kModeTrack) || idx >= d.f.H * d.f.W) return;
-  dilate_px(d.md, d.f.H, d.f.W, d.mask_out, idx);
-}
-
-constexpr int kFFW = 32, kFFH = 16;  // flood-fill tile (one thread per pixel)
-constexpr int kFFThreads = kFFW * kFFH;
-
-__device__ __forceinline__ bool ff_edge(unsigned Dsrc, unsigned Ddst, long long theta_ppm) {
-  const long long diff = Dsrc > Ddst ? (long long)(Dsrc - Ddst) : (long long)(Ddst - Dsrc);
-  return diff * 1000000ll < theta_ppm * (long long)Dsrc;
-}
-
-// ff words: [0] barrier count, [1] barrier generation, [2 + s] changed in sweep s
-// Run by a group of G CTAs, this one being number lb of the group.
-__device__ void floodfill_body(uint8_t* md, const uint16_t* __restrict__ depth, int H, int W, long long theta_ppm,
-                               unsigned* ff, int max_sweeps, unsigned* status, long long spin_limit,
-                               unsigned bar_extra, int lb, int G) {
-  __shared__ uint8_t sm[kFFH + 2][kFFW + 2];
-  __shared__ uint16_t sd[kFFH + 2][kFFW + 2];
-  const int tiles_x = (W + kFFW - 1) / kFFW, tiles_y = (H + kFFH - 1) / kFFH;
-  const int ntiles = tiles_x * tiles_y;
-  const int tx = threadIdx.x % kFFW, ty = threadIdx.x / kFFW;
-  unsigned* bar = ff;
-  unsigned* changed = ff + 2;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    for (int tile = lb; tile < ntiles; tile += G) {
-      const int u0 = (tile % tiles_x) * kFFW, v0 = (tile / tiles_x) * kFFH;
-      // tile + 1-pixel halo into shared memory
-      for (int i = threadIdx.x; i < (kFFH + 2) * (kFFW + 2); i += kFFThreads) {
-        const int hy = i / (kFFW + 2), hx = i % (kFFW + 2);
-        const int u = u0 + hx - 1, v = v0 + hy - 1;
-        const bool in = u >= 0 && u < W && v >= 0 && v < H;
-        sm[hy][hx] = in ? *(volatile uint8_t*)(md + v * W + u) : 0;
-        sd[hy][hx] = in ? __ldg(depth + v * W + u) : 0;
+  if (__syncthreads_or(some) && threadIdx.x == 0) atomicExch(d.ff + 6, 1u);
+  bool ok = grid_barrier(d.ff + 1, G, d.status, d.spin_limit, d.bar_extra);
+  const bool any = ok && *(volatile unsigned*)(d.ff + 6) != 0u;
+  bool settled = !any;
+  for (int sweep = 0; ok && !settled && sweep < d.max_sweeps; ++sweep) {
+    bool grew = false;
+    for (int reg = lb; reg < nreg; reg += G) {
+      const int tx = reg % regs_x * kFillTx + wx, ty = reg / regs_x * kFillTy + wy, tile = tile_at(tx, ty);
+      if (!resident && tile >= 0) {
+        t.m = __ldcg(words(tile) + kMPlane + lane);
+        load_planes(tile, ty, t);
       }
+      if (tile < 0) t = Tile{0u, 0u, 0u, 0u, 0u};
+      // facing borders of the tiles around the region (as of the last barrier)
+      unsigned top = 0u, bottom = 0u, left = 0u, right = 0u;
+      if (tile >= 0) {
+        if (wy == 0) top = border_word(tile_at(tx, ty - 1), 1);
+        if (wy == kFillTy - 1) bottom = border_word(tile_at(tx, ty + 1), 0);
+        if (wx == 0) left = border_word(tile_at(tx - 1, ty), 3);
+        if (wx == kFillTx - 1) right = border_word(tile_at(tx + 1, ty), 2);
+      }
+      const unsigned before = t.m;
+      int par = 0;
+      uint4 b = border_of(t.m);
+      __syncthreads();  // the last region's exchange has been read
+      if (lane == 0) sb[0][warp] = b;
       __syncthreads();
-      const int u = u0 + tx, v = v0 + ty;
-      const bool inside = u < W && v < H;
-      bool grew = false;
-      for (int it = 0; it < kFFThreads; ++it) {
-        int c = 0;
-        if (inside && !sm[ty + 1][tx + 1]) {
-          const unsigned Dp = sd[ty + 1][tx + 1];
-          if ((sm[ty + 1][tx] && ff_edge(sd[ty + 1][tx], Dp, theta_ppm)) ||
-              (sm[ty + 1][tx + 2] && ff_edge(sd[ty + 1][tx + 2], Dp, theta_ppm)) ||
-              (sm[ty][tx + 1] && ff_edge(sd[ty][tx + 1], Dp, theta_ppm)) ||
-              (sm[ty + 2][tx + 1] && ff_edge(sd[ty + 2][tx + 1], Dp, theta_ppm))) {
-            sm[ty + 1][tx + 1] = 1;
-            grew = true;
-            c = 1;
-          }
-        }
-        if (!__syncthreads_or(c)) break;
+      for (;;) {  // at most once per pixel of the region: each round but the last adds one
+        const unsigned was = t.m;
+        if (wy > 0) top = sb[par][warp - kFillTx].y;
+        if (wy < kFillTy - 1) bottom = sb[par][warp + kFillTx].x;
+        if (wx > 0) left = sb[par][warp - 1].w;
+        if (wx < kFillTx - 1) right = sb[par][warp + 1].z;
+        if (lane == 0) t.m |= t.down & top;
+        if (lane == 31) t.m |= t.up & bottom;
+        t.m |= (left >> lane) & t.right & 1u;
+        t.m |= (((right >> lane) & t.left_r) & 1u) << 31;  // (bit 0 of the reversed plane is column 31)
+        if (__any_sync(0xffffffffu, t.m != 0u)) t.m = settle(t, lane);
+        b = border_of(t.m);
+        par ^= 1;
+        if (lane == 0) sb[par][warp] = b;
+        if (!__syncthreads_or(t.m != was)) break;
       }
-      if (grew) md[v * W + u] = 1;
-      if (__syncthreads_or(grew) && threadIdx.x == 0) atomicExch(changed + sweep, 1u);
+      if (tile >= 0 && __any_sync(0xffffffffu, t.m != before)) {
+        grew = true;
+        put_border(tile, b);
+        if (!resident) __stcg(words(tile) + kMPlane + lane, t.m);
+      }
     }
-    if (!grid_barrier(bar, G, status, spin_limit, bar_extra)) return;
-    if (*(volatile unsigned*)(changed + sweep) == 0u) return;
+    if (__syncthreads_or(grew) && threadIdx.x == 0) atomicExch(d.ff + 3 + sweep % 3, 1u);
+    ok = grid_barrier(d.ff + 1, G, d.status, d.spin_limit, d.bar_extra);
+    if (!ok) break;
+    settled = changed[sweep % 3] == 0u;
+    // this sweep's predecessor's flag was read before the barrier; it serves
+    // the sweep after next
+    if (lb == 0 && threadIdx.x == 0) changed[(sweep + 2) % 3] = 0u;
   }
-  if (lb == 0 && threadIdx.x == 0) atomicOr(status, ST_NOT_CONVERGED);
+  if (ok && !settled && lb == 0 && threadIdx.x == 0) atomicOr(d.status, ST_NOT_CONVERGED);
+  // dilation, from the tiles and the facing borders of the eight around each
+  // (16-byte stores where every row starts on a 16-byte boundary)
+  const bool wide_stores = (W & 15) == 0 && (reinterpret_cast<uintptr_t>(d.mask_out) & 15) == 0;
+  for (int reg = lb; reg < nreg; reg += G) {
+    const int tx = reg % regs_x * kFillTx + wx, ty = reg / regs_x * kFillTy + wy, tile = tile_at(tx, ty);
+    if (tile < 0) continue;
+    unsigned out = 0u;
+    if (any) {
+      if (!resident) t.m = __ldcg(words(tile) + kMPlane + lane);
+      const unsigned left = border_word(tile_at(tx - 1, ty), 3), right = border_word(tile_at(tx + 1, ty), 2);
+      const unsigned wide = t.m | (t.m << 1) | (t.m >> 1) | ((left >> lane) & 1u) | (((right >> lane) & 1u) << 31);
+      auto wide_row = [&](int y, int k) {  // the row next to the tile, widened
+        const unsigned w = border_word(tile_at(tx, y), k);
+        return w | (w << 1) | (w >> 1) | (border_word(tile_at(tx - 1, y), k) >> 31) |
+               (border_word(tile_at(tx + 1, y), k) << 31);
+      };
+      const unsigned above = wide_row(ty - 1, 1), below = wide_row(ty + 1, 0);
+      const unsigned wu = __shfl_up_sync(0xffffffffu, wide, 1), wd = __shfl_down_sync(0xffffffffu, wide, 1);
+      out = wide | (lane == 0 ? above : wu) | (lane == 31 ? below : wd);
+    }
+    const int y = ty * 32 + lane;
+    if (wide_stores && tx * 32 + 32 <= W) {
+      // each lane its row's 32 bytes: a multiplication spreads four bits over four bytes
+      unsigned q[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = (((out >> (4 * k)) & 15u) * 0x00204081u) & 0x01010101u;
+      if (y < H) {
+        uint4* o = reinterpret_cast<uint4*>(d.mask_out + (size_t)y * W + tx * 32);
+        o[0] = make_uint4(q[0], q[1], q[2], q[3]);
+        o[1] = make_uint4(q[4], q[5], q[6], q[7]);
+      }
+    } else {
+      const int u = tx * 32 + lane;
+#pragma unroll 8
+      for (int r = 0; r < 32; ++r) {
+        const unsigned row = __shfl_sync(0xffffffffu, out, r);
+        const int v = ty * 32 + r;
+        if (u < W && v < H) d.mask_out[(size_t)v * W + u] = (uint8_t)((row >> lane) & 1u);
+      }
+    }
+  }
 }
 
-__global__ void __launch_bounds__(kFFThreads) k_floodfill(uint8_t* md, const uint16_t* __restrict__ depth, int H,
-                                                           int W, long long theta_ppm, unsigned* ff, int max_sweeps,
-                                                           unsigned* status, const int* gate, long long spin_limit,
-                                                           unsigned bar_extra) {
-  if (gated_off(gate, kModeTrack)) return;  // uniform over the grid: before any barrier
-  floodfill_body(md, depth, H, W, theta_ppm, ff, max_sweeps, status, spin_limit, bar_extra, blockIdx.x, gridDim.x);
-}
+__global__ void __launch_bounds__(kFillThreads) k_mask_fill(FillDesc d) { mask_fill_body(d, blockIdx.x, gridDim.x); }
 
-// The flood fills of several streams in one cooperative launch: CTA b runs
-// stream cta_stream[b] (-1: none) as member b - first[s] of its group (the
-// CTA maps of the batched registration).  Groups never wait on each other.
-__global__ void __launch_bounds__(kFFThreads) k_floodfill_batch(const FloodDesc* __restrict__ descs,
-                                                                 const int* __restrict__ cta_stream,
-                                                                 const int* __restrict__ first) {
+// The same for several streams in one cooperative launch: CTA b runs stream
+// cta_stream[b] (-1: none) as member b - first[s] of its group (the CTA maps
+// of the batched registration).  Groups never wait on each other.
+__global__ void __launch_bounds__(kFillThreads) k_mask_fill_batch(const FillDesc* __restrict__ descs,
+                                                                  const int* __restrict__ cta_stream,
+                                                                  const int* __restrict__ first) {
   const int s = cta_stream[blockIdx.x];
   if (s < 0) return;
-  const FloodDesc d = descs[s];
-  floodfill_body(d.md, d.depth, d.H, d.W, d.theta_ppm, d.ff, d.max_sweeps, d.status, d.spin_limit, d.bar_extra,
-                 blockIdx.x - first[s], first[s + 1] - first[s]);
+  mask_fill_body(descs[s], blockIdx.x - first[s], first[s + 1] - first[s]);
 }
 
 }  // namespace
 
-rf_status launch_mask_pre(rf_volume* vol, const DevFrame& f, const double* T, cudaStream_t st) {
-  const int n = f.H * f.W;
-  const int blocks = (n + 255) / 256;
-  rf_status s = check_cuda(vol, cudaMemsetAsync(vol->d_guard, 0, sizeof(unsigned), st), "guard reset");
-  if (s != RF_OK) return s;
+static rf_status launch_seeds(rf_volume* vol, const DevFrame& f, const double* T, unsigned* tiles, unsigned* guard,
+                              cudaStream_t st) {
+  const int blocks = seed_blocks(f.H, f.W);
   if (vol->p.storage == RF_STORAGE_FP16)
-    k_seeds<RF_STORAGE_FP16><<<seed_blocks(n), kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T, vol->d_seeds,
-                                                                       vol->d_guard, vol->d_pxcache);
+    k_seeds<RF_STORAGE_FP16><<<blocks, kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T, tiles, guard, vol->d_pxcache);
   else
-    k_seeds<RF_STORAGE_FP32><<<seed_blocks(n), kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T, vol->d_seeds,
-                                                                       vol->d_guard, vol->d_pxcache);
-  k_erode<<<blocks, 256, 0, st>>>(vol->d_seeds, f.H, f.W, vol->d_md, f.gate);
-  s = check_cuda(vol, cudaMemsetAsync(vol->d_ff, 0, sizeof(unsigned) * (2 + vol->p.max_ff_sweeps), st),
-                 "flood-fill reset");
-  if (s != RF_OK) return s;
-  return check_cuda(vol, cudaGetLastError(), "mask launch");
+    k_seeds<RF_STORAGE_FP32><<<blocks, kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T, tiles, guard, vol->d_pxcache);
+  return check_cuda(vol, cudaGetLastError(), "seeds launch");
 }
 
-rf_status launch_mask_ff(rf_volume* vol, const DevFrame& f, cudaStream_t st) {
-  const int ntiles = ((f.W + kFFW - 1) / kFFW) * ((f.H + kFFH - 1) / kFFH);
-  const int grid = ntiles < vol->ff_grid ? ntiles : vol->ff_grid;
+static rf_status launch_coop(rf_volume* vol, const void* fn, int grid, void** args, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kFFThreads);
+  cfg.blockDim = dim3(kFillThreads);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return check_cuda(vol,
-                    cudaLaunchKernelEx(&cfg, k_floodfill, vol->d_md, f.depth, f.H, f.W, vol->dp.theta_ppm, vol->d_ff,
-                                       vol->p.max_ff_sweeps, vol->d_status, f.gate, vol->wait_spins,
-                                       vol->wait_extra),
-                    "flood-fill launch");
+  return check_cuda(vol, cudaLaunchKernelExC(&cfg, fn, args), "flood-fill launch");
 }
 
-MaskDesc make_mask_desc(rf_volume* vol, const DevFrame& f, const double* T, uint8_t* mask_out) {
-  MaskDesc d;
-  d.v = vol->dv;
-  d.f = f;
-  d.p = vol->dp;
-  d.T = T;
-  d.seeds = vol->d_seeds;
-  d.guard = vol->d_guard;
-  d.md = vol->d_md;
+static rf_status launch_fill(rf_volume* vol, FillDesc d, cudaStream_t st) {
+  const int rx = (d.W + 32 * kFillTx - 1) / (32 * kFillTx), ry = (d.H + 32 * kFillTy - 1) / (32 * kFillTy);
+  void* args[] = {&d};
+  return launch_coop(vol, (const void*)k_mask_fill, rx * ry < vol->ff_grid ? rx * ry : vol->ff_grid, args, st);
+}
+
+FillDesc make_fill_desc(rf_volume* vol, const DevFrame& f, uint8_t* mask_out) {
+  FillDesc d;
   d.mask_out = mask_out;
-  d.pxcache = vol->d_pxcache;
-  return d;
-}
-
-rf_status launch_mask_pre_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_npix, cudaStream_t st) {
-  const dim3 grid((unsigned)((max_npix + 255) / 256), (unsigned)n);
-  const dim3 sgrid((unsigned)seed_blocks(max_npix), (unsigned)n);
-  if (vol->p.storage == RF_STORAGE_FP16)
-    k_seeds_batch<RF_STORAGE_FP16><<<sgrid, kSeedThreads, 0, st>>>(descs);
-  else
-    k_seeds_batch<RF_STORAGE_FP32><<<sgrid, kSeedThreads, 0, st>>>(descs);
-  k_erode_batch<<<grid, 256, 0, st>>>(descs);
-  return check_cuda(vol, cudaGetLastError(), "batched mask launch");
-}
-
-rf_status launch_mask_post_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_npix, cudaStream_t st) {
-  k_dilate_batch<<<dim3((unsigned)((max_npix + 255) / 256), (unsigned)n), 256, 0, st>>>(descs);
-  return check_cuda(vol, cudaGetLastError(), "batched mask launch");
-}
-
-rf_status launch_mask_post(rf_volume* vol, const DevFrame& f, uint8_t* mask_out, cudaStream_t st) {
-  const int n = f.H * f.W;
-  k_dilate<<<(n + 255) / 256, 256, 0, st>>>(vol->d_md, f.H, f.W, mask_out, f.gate);
-  return check_cuda(vol, cudaGetLastError(), "mask launch");
-}
-
-rf_status launch_mask(rf_volume* vol, const DevFrame& f, const double* T, uint8_t* mask_out, cudaStream_t st) {
-  rf_status s = launch_mask_pre(vol, f, T, st);
-  if (s == RF_OK) s = launch_mask_ff(vol, f, st);
-  if (s == RF_OK) s = launch_mask_post(vol, f, mask_out, st);
-  return s;
-}
-
-FloodDesc make_flood_desc(rf_volume* vol, const DevFrame& f) {
-  FloodDesc d;
-  d.md = vol->d_md;
-  d.depth = f.depth;
+  d.tiles = vol->d_tiles;
   d.H = f.H;
   d.W = f.W;
-  d.theta_ppm = vol->dp.theta_ppm;
   d.ff = vol->d_ff;
   d.max_sweeps = vol->p.max_ff_sweeps;
   d.status = vol->d_status;
@@ -427,40 +524,64 @@ FloodDesc make_flood_desc(rf_volume* vol, const DevFrame& f) {
   return d;
 }
 
-rf_status launch_floodfill_batch(rf_volume* vol, const FloodDesc* descs, const int* cta_stream, const int* first,
-                                 int total_ctas, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(total_ctas);
-  cfg.blockDim = dim3(kFFThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return check_cuda(vol, cudaLaunchKernelEx(&cfg, k_floodfill_batch, descs, cta_stream, first),
-                    "batched flood-fill launch");
+rf_status launch_mask(rf_volume* vol, const DevFrame& f, const double* T, uint8_t* mask_out, cudaStream_t st) {
+  rf_status s = check_cuda(vol, cudaMemsetAsync(vol->d_ff, 0, sizeof(unsigned) * kFillWords, st), "mask words reset");
+  if (s == RF_OK) s = launch_seeds(vol, f, T, vol->d_tiles, vol->d_guard, st);
+  if (s == RF_OK) s = launch_fill(vol, make_fill_desc(vol, f, mask_out), st);
+  return s;
 }
 
+MaskDesc make_mask_desc(rf_volume* vol, const DevFrame& f, const double* T) {
+  MaskDesc d;
+  d.v = vol->dv;
+  d.f = f;
+  d.p = vol->dp;
+  d.T = T;
+  d.tiles = vol->d_tiles;
+  d.guard = vol->d_guard;
+  d.pxcache = vol->d_pxcache;
+  return d;
+}
+
+rf_status launch_seeds_batch(rf_volume* vol, const MaskDesc* descs, int n, int max_blocks, cudaStream_t st) {
+  const dim3 grid((unsigned)max_blocks, (unsigned)n);
+  if (vol->p.storage == RF_STORAGE_FP16)
+    k_seeds_batch<RF_STORAGE_FP16><<<grid, kSeedThreads, 0, st>>>(descs);
+  else
+    k_seeds_batch<RF_STORAGE_FP32><<<grid, kSeedThreads, 0, st>>>(descs);
+  return check_cuda(vol, cudaGetLastError(), "batched seeds launch");
+}
+
+rf_status launch_fill_batch(rf_volume* vol, const FillDesc* descs, const int* cta_stream, const int* first,
+                            int total_ctas, cudaStream_t st) {
+  void* args[] = {(void*)&descs, (void*)&cta_stream, (void*)&first};
+  return launch_coop(vol, (const void*)k_mask_fill_batch, total_ctas, args, st);
+}
+
+int mask_seed_blocks(int H, int W) { return seed_blocks(H, W); }
+
 int floodfill_max_grid(int device) {
-  int per_sm = 0, sms = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_floodfill, kFFThreads, 0);
+  int per_sm = 1 << 20, sms = 0;
+  for (const void* fn : {(const void*)k_mask_fill, (const void*)k_mask_fill_batch}) {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kFillThreads, 0);
+    per_sm = n < per_sm ? n : per_sm;
+  }
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   return per_sm * sms;
 }
 
 // ---------------------------------------------------------------------------
-// Mask without any allocation: the per-call scratch of rf_compute_mask (seed
-// image, flood-fill working mask, barrier words, per-sweep change flags and the
-// guard counter) lives in one file-scope device array instead of the buffers
+// Mask without any allocation: the per-call scratch of rf_compute_mask (the
+// flood fill's tiles, barrier words, change flags and the guard counter) lives in one file-scope device array instead of the buffers
 // the volume owns.  Every GPU that loads this library holds the array (about
-// 1.9 MB) until the process exits.
+// 0.9 MB) until the process exits.
 // ---------------------------------------------------------------------------
 constexpr int kNoAllocMaxPixels = 1280 * 720;  // largest frame: 921,600 pixels
+constexpr int kNoAllocMaxTiles = 1152;          // of frames that size with sides up to 8,192
 constexpr int kNoAllocMaxSweeps = 4096;         // flood-fill sweep bound of this entry point
-constexpr size_t kNoAllocWordsOff = 2 * (size_t)kNoAllocMaxPixels;  // multiple of 256
-constexpr size_t kNoAllocWords = 2 + kNoAllocMaxSweeps + 1;         // barrier, change flags, guard count
-constexpr size_t kNoAllocBytes = kNoAllocWordsOff + sizeof(unsigned) * kNoAllocWords;
+constexpr size_t kNoAllocWordsOff = sizeof(unsigned) * kNoAllocMaxTiles * kFillTileWords;
+constexpr size_t kNoAllocBytes = kNoAllocWordsOff + sizeof(unsigned) * kFillWords;
 
 static __device__ __align__(256) unsigned char g_mask_scratch[kNoAllocBytes];
 
@@ -508,39 +629,16 @@ extern "C" rf_status rf_compute_mask_noalloc(rf_volume* vol, const rf_frame* fra
   cudaError_t e;
   unsigned char* base = static_cast<unsigned char*>(mask_scratch_address(vol->device, &e));
   if (!base) return check_cuda(vol, e, "cudaGetSymbolAddress(mask scratch)");
-  uint8_t* seeds = base;
-  uint8_t* md = base + kNoAllocMaxPixels;
   unsigned* ff = reinterpret_cast<unsigned*>(base + kNoAllocWordsOff);
-  unsigned* guard = ff + 2 + kNoAllocMaxSweeps;
-  const int sweeps = vol->p.max_ff_sweeps < kNoAllocMaxSweeps ? vol->p.max_ff_sweeps : kNoAllocMaxSweeps;
   cudaStream_t st = (cudaStream_t)stream;
   const DevFrame f = make_dev_frame(frame);
-  const int n = f.H * f.W;
-  const int blocks = (n + 255) / 256;
   // the array keeps the previous call's contents: zero the words that count
-  if ((s = check_cuda(vol, cudaMemsetAsync(ff, 0, sizeof(unsigned) * kNoAllocWords, st), "scratch clear"))) return s;
-  if (vol->p.storage == RF_STORAGE_FP16)
-    k_seeds<RF_STORAGE_FP16><<<seed_blocks(n), kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T_dev, seeds, guard,
-                                                                       vol->d_pxcache);
-  else
-    k_seeds<RF_STORAGE_FP32><<<seed_blocks(n), kSeedThreads, 0, st>>>(vol->dv, f, vol->dp, T_dev, seeds, guard,
-                                                                       vol->d_pxcache);
-  k_erode<<<blocks, 256, 0, st>>>(seeds, f.H, f.W, md, nullptr);
-  const int ntiles = ((f.W + kFFW - 1) / kFFW) * ((f.H + kFFH - 1) / kFFH);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ntiles < vol->ff_grid ? ntiles : vol->ff_grid);
-  cfg.blockDim = dim3(kFFThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if ((s = check_cuda(vol, cudaLaunchKernelEx(&cfg, k_floodfill, md, f.depth, f.H, f.W, vol->dp.theta_ppm, ff,
-                                              sweeps, vol->d_status, (const int*)nullptr, vol->wait_spins,
-                                              vol->wait_extra),
-                      "flood-fill launch")))
-    return s;
-  k_dilate<<<blocks, 256, 0, st>>>(md, f.H, f.W, mask_dev, nullptr);
-  return check_cuda(vol, cudaGetLastError(), "mask launch");
+  if ((s = check_cuda(vol, cudaMemsetAsync(ff, 0, sizeof(unsigned) * kFillWords, st), "scratch clear"))) return s;
+  unsigned* tiles = reinterpret_cast<unsigned*>(base);
+  if ((s = launch_seeds(vol, f, T_dev, tiles, ff, st))) return s;
+  FillDesc d = make_fill_desc(vol, f, mask_dev);
+  d.tiles = tiles;
+  d.ff = ff;
+  d.max_sweeps = d.max_sweeps < kNoAllocMaxSweeps ? d.max_sweeps : kNoAllocMaxSweeps;
+  return launch_fill(vol, d, st);
 }

@@ -43,9 +43,8 @@ struct rf_volume {
   int reg_grid = 0;
 
   // mask scratch
-  uint8_t* d_seeds = nullptr;
-  uint8_t* d_md = nullptr;     // M_D during the flood fill
-  unsigned* d_ff = nullptr;    // barrier words + per-sweep change flags
+  unsigned* d_tiles = nullptr;  // raw mask, join conditions and flood fill, as bits in tiles (kFillTileWords each)
+  unsigned* d_ff = nullptr;     // guard count, barrier words, change flags (kFillWords)
   int ff_grid = 0;
 
   // integration scratch
@@ -61,7 +60,7 @@ struct rf_volume {
   double* d_T = nullptr;        // [3][16]: T_in, T_first, T_second
   rf_track_info* d_info = nullptr;
 
-  unsigned* d_guard = nullptr;  // FP64 re-evaluated seed count of the last mask
+  unsigned* d_guard = nullptr;  // FP64 re-evaluated seed count of the last mask (d_ff[0])
   unsigned long long* d_pxcache = nullptr;  // per pixel: block key << 22 | pool of its last sample
 
   // profiling: events recorded around the stages of the whole-frame calls
