@@ -130,7 +130,7 @@ typedef struct rf_profile {
   int64_t candidates;        /* frustum candidate blocks of the last integration */
   int64_t updated_voxels;    /* voxels updated by the last integration */
   int64_t new_blocks;        /* blocks allocated by the last integration */
-  int64_t guard_pixels;      /* mask seeds decided by the FP64 re-evaluation in the last mask */
+  int64_t guard_pixels;      /* mask seeds (ray samples) that FP32 left open in the last mask (virtual depth) */
 } rf_profile;
 
 typedef struct rf_volume rf_volume;

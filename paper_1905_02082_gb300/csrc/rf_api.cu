@@ -58,6 +58,10 @@ DevFrame make_dev_frame(const rf_frame* f) {
   // the image extent around the principal point (see the integration kernel)
   d.amb_u = (float)(4.0 * (6e-7 * 2.0 * (f->width + std::fabs(f->cx)) + 2.5e-4));
   d.amb_v = (float)(4.0 * (6e-7 * 2.0 * (f->height + std::fabs(f->cy)) + 2.5e-4));
+  d.cx_lo = (float)(f->cx - (double)d.cx);
+  d.cy_lo = (float)(f->cy - (double)d.cy);
+  d.ifx_lo = (float)(1.0 / f->fx - (double)d.ifx);
+  d.ify_lo = (float)(1.0 / f->fy - (double)d.ify);
   d.depth = f->depth;
   d.rgb = f->rgb;
   d.gate = nullptr;
@@ -177,7 +181,9 @@ rf_status volume_buffers(rf_volume* vol, const rf_params* p, int64_t n_buckets, 
       (s = A(&vol->d_dmask, npix, "masked depth")) ||
       // (a registration keeps its pixel records in the candidate list's memory:
       // the two never run at the same time on one volume)
-      (s = A(&vol->d_cand, std::max((size_t)p->max_candidates, reg_records(p, max_width, max_height)), "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
+      // (virtual depth keeps its hole list there: two ints per pixel)
+      (s = A(&vol->d_cand, std::max({(size_t)p->max_candidates, reg_records(p, max_width, max_height), npix / 2 + 1}),
+             "candidates / pixel records")) || (s = A(&vol->d_depth, npix, "depth staging")) ||
       (s = A(&vol->d_rgb, npix * 3, "rgb staging")) || (s = A(&vol->d_mask, npix, "mask staging")) ||
       (s = A(&vol->d_T, 48, "poses")) || (s = A(&vol->d_info, 1, "info")) ||
       (s = A(&vol->d_pxcache, npix, "pixel block cache")))
@@ -212,6 +218,11 @@ DevParams derive(const rf_params& p) {
   d.theta_ppm = llround(p.theta * 1e6);
   d.storage = p.storage;
   d.inv_tau = (float)(1.0 / p.trunc);
+  d.inv_voxel_lo = (float)(1.0 / p.voxel_size - (double)d.inv_voxel);
+  d.inv_depth_scale_lo = (float)(1.0 / p.depth_scale - (double)d.inv_depth_scale);
+  d.z_near_lo = (float)(p.z_near - (double)d.z_near);
+  d.half_voxel = (float)(p.voxel_size * 0.5);
+  d.half_voxel_lo = (float)(p.voxel_size * 0.5 - (double)d.half_voxel);
   d.du_tick = (unsigned)(d.du_um * 1024);
   return d;
 }

@@ -66,6 +66,8 @@ struct DevParams {
   long long theta_ppm;
   int storage;    // voxel storage mode (0: FP32, 1: compact FP16)
   float inv_tau;  // 1 / tau (FP16 encoding of F / tau)
+  // what the floats above (or their reciprocals) lack of the doubles, as floats
+  float inv_voxel_lo, inv_depth_scale_lo, z_near_lo, half_voxel, half_voxel_lo;
   unsigned du_tick;  // ticks (2^-10 um) per raw depth unit
 };
 
@@ -80,6 +82,8 @@ struct DevFrame {
   // float pixel estimates closer than this to a rounding boundary are decided
   // by the exact integer path (4x the bound on the estimate's error)
   float amb_u, amb_v;
+  // what cx, cy, ifx and ify lack of the doubles, as floats
+  float cx_lo, cy_lo, ifx_lo, ify_lo;
   const uint16_t* depth;
   const uint8_t* rgb;
   // batches only: the stream's per-call mode (kMode*), read by every mask and
@@ -264,6 +268,67 @@ __device__ __forceinline__ unsigned rgb_i8(unsigned c) {
   const unsigned s = __dp2a_hi(722u, c & 0x00FFFFFFu, __dp2a_lo(2126u | (7152u << 16), c, 0u));
   return (254u * s + 1275000u) / 2550000u;
 }
+
+// ---------------------------------------------------------------------------
+// Float pairs: an unevaluated sum h + l, about 46 bits, in FP32 instructions.
+// On GB300 a warp's FP64 instruction holds the SM's FP64 pipe for 16 cycles
+// and returns after 300-400; a decision that FP32 leaves open is therefore
+// taken in float pairs first, and in FP64 only when those leave it open too.
+// Sums are accurate to 2^-44 of their operands' magnitudes, products to 2^-44
+// relative.
+// ---------------------------------------------------------------------------
+struct FF {
+  float h, l;
+};
+__device__ __forceinline__ FF ff_norm(float h, float l) {  // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return FF{s, __fadd_rn(l, -__fadd_rn(s, -h))};
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b) {
+  const float s = __fadd_rn(a.h, b.h), bb = __fadd_rn(s, -a.h);
+  const float e = __fadd_rn(__fadd_rn(a.h, -__fadd_rn(s, -bb)), __fadd_rn(b.h, -bb));
+  return ff_norm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
+  return ff_norm(p, e);
+}
+
+// Lattice cell (k, fr) in float pairs of the camera point at pixel (u, vv) and
+// depth z: false when it may lie in another cell (within the bound of a
+// boundary).  T: the pose's 12 entries (rows R | t) as float pairs.  Against
+// the FP64 evaluation q is within 2^-40 of the magnitudes that enter it (16
+// times the pairs' error), and fr, rounded to a float, within 2^-23 more.
+__device__ __forceinline__ bool cell_ff(const DevFrame& f, const DevParams& p, const FF* T, int u, int vv, FF z, int k[3],
+                                        float fr[3]) {
+  const FF iv = {p.inv_voxel, p.inv_voxel_lo};
+  const FF x = ff_mul(ff_mul(ff_add(FF{(float)u, 0.0f}, FF{-f.cx, -f.cx_lo}), FF{f.ifx, f.ifx_lo}), z);
+  const FF y = ff_mul(ff_mul(ff_add(FF{(float)vv, 0.0f}, FF{-f.cy, -f.cy_lo}), FF{f.ify, f.ify_lo}), z);
+  const float mag = (fabsf(x.h) + fabsf(y.h) + fabsf(z.h) + fabsf(T[3].h) + fabsf(T[7].h) + fabsf(T[11].h)) * p.inv_voxel;
+  const float eps = mag * 9.094947e-13f + 2.3841858e-07f;  // 2^-40, 2^-22
+  bool sure = mag < 8.0f * kMaxCoord - 2.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const FF q = ff_mul(ff_add(ff_add(ff_mul(T[4 * i], x), ff_mul(T[4 * i + 1], y)),
+                               ff_add(ff_mul(T[4 * i + 2], z), T[4 * i + 3])),
+                        iv);
+    float fl = floorf(q.h), r = (q.h - fl) + q.l;  // (the difference is exact)
+    if (r < 0.0f) {
+      fl -= 1.0f;
+      r += 1.0f;
+    } else if (r >= 1.0f) {
+      fl += 1.0f;
+      r -= 1.0f;
+    }
+    k[i] = (int)fl;
+    fr[i] = r;
+    sure = sure && r > eps && r < 1.0f - eps;
+  }
+  return sure;
+}
+constexpr float kFrErrFF = 4.7683716e-07f;  // bound on |fr - FP64 fr| of a sure cell (2^-21)
 
 // FP64 lerp in the oracle's operation order (no contraction).
 __device__ __forceinline__ double lerp_rn(double a, double b, double t) {
@@ -488,7 +553,10 @@ rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const int*
 // erosion, flood fill and dilation of several streams in one cooperative
 // launch (the batches' CTA maps; total_ctas must not exceed floodfill_max_grid)
 constexpr int kFillTileWords = 6 * 32 + 4;  // global memory of one 32 x 32 tile
-constexpr int kFillWords = 8;  // guard count, barrier (2), change flags (3), M_R not empty; zeroed per mask
+// words zeroed at the start of a mask or a virtual-depth call: [0] guard count;
+// mask: [1, 2] barrier, [3..5] change flags, [6] M_R not empty; virtual depth:
+// [8] holes, [9..14] bounds of the allocated blocks
+constexpr int kFillWords = 16;
 struct FillDesc {
   uint8_t* mask_out;
   unsigned* tiles;  // kFillTileWords per tile, written by the seeds

@@ -5,7 +5,8 @@
 //                warp per 32 pixels of a row, written as bits.  The
 //                decision is exact: the FP32 evaluation carries an error bound;
 //                when the lattice cell or the comparison is within it, the pixel
-//                is re-evaluated in FP64 with a fixed operation order and no
+//                is re-evaluated in float pairs with a far smaller bound, and
+//                within that one in FP64 with a fixed operation order and no
 //                contraction (__d*_rn), the order the FP64 oracle uses.  The
 //                warps also write the pixels' join conditions of Alg. 1, as bits.
 //   k_mask_fill  the rest, in one cooperative launch: M_R = 3x3 erosion of the raw
@@ -55,13 +56,35 @@ __device__ double residual_fp64(const DevVol& v, const DevFrame& f, const DevPar
   return __dmul_rn(V, V);
 }
 
+// Seed decision from the cell's corners and the position in it, known within
+// eps_q: 0 or 1, or 2 when the comparison lies within the error bound.
+__device__ __forceinline__ int seed_of(const DevParams& p, const float F[8], const float fr[3], float eps_q) {
+  const float t = p.gamma_tau2_f;
+  const float c00 = F[0] * (1.0f - fr[0]) + F[1] * fr[0], c10 = F[2] * (1.0f - fr[0]) + F[3] * fr[0];
+  const float c01 = F[4] * (1.0f - fr[0]) + F[5] * fr[0], c11 = F[6] * (1.0f - fr[0]) + F[7] * fr[0];
+  const float c0 = c00 * (1.0f - fr[1]) + c10 * fr[1], c1 = c01 * (1.0f - fr[1]) + c11 * fr[1];
+  const float V = fminf(fmaxf(c0 * (1.0f - fr[2]) + c1 * fr[2], -p.tau), p.tau);
+  float fmn = F[0], fmx = F[0], fab = fabsf(F[0]);
+#pragma unroll
+  for (int n = 1; n < 8; ++n) {
+    fmn = fminf(fmn, F[n]);
+    fmx = fmaxf(fmx, F[n]);
+    fab = fmaxf(fab, fabsf(F[n]));
+  }
+  // + the gap between the float and double truncation bounds (<= 2^-24 tau)
+  const float dV = 3.0f * (fmx - fmn) * eps_q + fab * 1.9073486328125e-06f + p.tau * 5.9604645e-08f;
+  const float r = V * V;
+  const float dr = 2.0f * fabsf(V) * dV + dV * dV + r * 2.384185791015625e-07f;  // 2^-22
+  if (fabsf(r - t) <= 2.0f * dr + t * 2.384185791015625e-07f) return 2;
+  return r > t ? 1 : 0;
+}
+
 // Seed decision of one valid pixel in FP32 with an error bound: 0 or 1, or
 // 2 when the lattice cell or the comparison lies within the bound (the pixel
 // is then decided in FP64).  Rf: the pose as floats (R row-major, then t).
 template <int ST>
 __device__ __forceinline__ int seed_fp32(const DevVol& v, const DevFrame& f, const DevParams& p, const float* Rf, int u,
                                          int vv, unsigned raw, unsigned long long cached) {
-  const float t = p.gamma_tau2_f;
   const float D = (float)raw * p.inv_depth_scale;
   const float x = ((float)u - f.cx) * f.ifx * D, y = ((float)vv - f.cy) * f.ify * D;
   float q[3], fr[3];
@@ -89,23 +112,19 @@ __device__ __forceinline__ int seed_fp32(const DevVol& v, const DevFrame& f, con
   float F[8];
   // an unambiguous cell with a missing corner is invalid in FP64 too: no seed
   if (!corners_cached<ST>(v, p, k[0], k[1], k[2], cached, F)) return 0;
-  const float c00 = F[0] * (1.0f - fr[0]) + F[1] * fr[0], c10 = F[2] * (1.0f - fr[0]) + F[3] * fr[0];
-  const float c01 = F[4] * (1.0f - fr[0]) + F[5] * fr[0], c11 = F[6] * (1.0f - fr[0]) + F[7] * fr[0];
-  const float c0 = c00 * (1.0f - fr[1]) + c10 * fr[1], c1 = c01 * (1.0f - fr[1]) + c11 * fr[1];
-  const float V = fminf(fmaxf(c0 * (1.0f - fr[2]) + c1 * fr[2], -p.tau), p.tau);
-  float fmn = F[0], fmx = F[0], fab = fabsf(F[0]);
-#pragma unroll
-  for (int n = 1; n < 8; ++n) {
-    fmn = fminf(fmn, F[n]);
-    fmx = fmaxf(fmx, F[n]);
-    fab = fmaxf(fab, fabsf(F[n]));
-  }
-  // + the gap between the float and double truncation bounds (<= 2^-24 tau)
-  const float dV = 3.0f * (fmx - fmn) * eps_q + fab * 1.9073486328125e-06f + p.tau * 5.9604645e-08f;
-  const float r = V * V;
-  const float dr = 2.0f * fabsf(V) * dV + dV * dV + r * 2.384185791015625e-07f;  // 2^-22
-  if (fabsf(r - t) <= 2.0f * dr + t * 2.384185791015625e-07f) return 2;
-  return r > t ? 1 : 0;
+  return seed_of(p, F, fr, eps_q);
+}
+
+// The same in float pairs.
+template <int ST>
+__device__ __forceinline__ int seed_ff(const DevVol& v, const DevFrame& f, const DevParams& p, const FF* T, int u, int vv,
+                                       unsigned raw) {
+  const FF D = ff_mul(FF{(float)raw, 0.0f}, FF{p.inv_depth_scale, p.inv_depth_scale_lo});
+  int k[3];
+  float fr[3], F[8];
+  if (!cell_ff(f, p, T, u, vv, D, k, fr)) return 2;
+  if (!corners_of<ST>(v, p, k[0], k[1], k[2], F)) return 0;
+  return seed_of(p, F, fr, kFrErrFF);
 }
 
 __device__ __forceinline__ bool may_join(unsigned from, unsigned to, long long theta_ppm) {
@@ -124,10 +143,10 @@ static_assert(kBorder + 4 == kFillTileWords, "tile layout");
 // Seeds and join conditions of the kSeedThreads / 32 * kSeedPx row words (32
 // pixels of a row, the first one's column a multiple of 32) of CTA `block`.
 // Every thread first loads its pixels' depths and cache entries, then decides
-// them in FP32; the ambiguous ones are queued in shared
-// memory and decided in FP64 afterwards, side by side by consecutive threads:
-// on GB300 the FP64 pipe is narrow, and a warp that takes the FP64 branch for
-// one of its lanes costs as much as one that takes it for all 32.
+// them in FP32; the ambiguous ones (~2 %, almost all for their lattice cell)
+// are queued in shared memory and decided in float pairs afterwards, side by
+// side by consecutive threads, and what that leaves open (one in thousands of
+// them) in FP64, whose chain alone took half the kernel's time.
 // The join conditions of Alg. 1 are decided here, where every SM has pixels and
 // the issue slots are idle (the lookups' latency bounds the kernel), and not in
 // the flood fill, which runs on few SMs (there they took 13 us of 640x480).
@@ -145,18 +164,17 @@ __device__ __forceinline__ void seeds_body(const DevVol& v, const DevFrame& f, c
                                            const double* __restrict__ T, unsigned* __restrict__ tiles,
                                            unsigned* guard_count, const unsigned long long* __restrict__ pxcache,
                                            int block) {
-  // pose and threshold converted once per CTA (conversions use the FP64 pipe)
+  // pose converted once per CTA (conversions use the FP64 pipe)
   __shared__ float sR[12];
-  __shared__ double s_t64;
   __shared__ unsigned short s_queue[kSeedWords * 32];
   __shared__ unsigned s_words[kSeedWords];
-  __shared__ int s_n;
+  __shared__ int s_n, s_open, s_last[kSeedThreads];
+  __shared__ FF s_T[12];
   if (threadIdx.x < 12) {
     const int i = threadIdx.x < 9 ? threadIdx.x / 3 : threadIdx.x - 9;
     const int j = threadIdx.x < 9 ? threadIdx.x % 3 : 3;
     sR[threadIdx.x] = (float)T[i * 4 + j];
   }
-  if (threadIdx.x == 12) s_t64 = __dmul_rn(__dmul_rn(p.gamma_d, p.tau_d), p.tau_d);
   if (threadIdx.x == 13) s_n = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -212,13 +230,41 @@ __device__ __forceinline__ void seeds_body(const DevVol& v, const DevFrame& f, c
       tile_word(w)[kRightPlane + 32 * lane] = x;
     }
   }
+  if (threadIdx.x < 12) {  // the pose in float pairs
+    const double t = T[threadIdx.x];
+    const float h = (float)t;
+    s_T[threadIdx.x] = FF{h, (float)(t - (double)h)};
+  }
   __syncthreads();
   const int n = s_n;
-  for (int i = threadIdx.x; i < n; i += kSeedThreads) {
-    const int local = s_queue[i] >> 5, bit = s_queue[i] & 31, w = word_of(local), row = w / rw;
-    const int u = (w - row * rw) * 32 + bit;
-    const double r64 = residual_fp64<ST>(v, f, p, T, u, row, __ldg(f.depth + row * f.W + u));
-    if (r64 >= 0.0 && r64 > s_t64) atomicOr(&s_words[local], 1u << bit);
+  // the ambiguous pixels in float pairs, then those that remain so in FP64
+  auto pixel_of = [&](int q, int& u, int& row) {
+    const int w = word_of(q >> 5);
+    row = w / rw;
+    u = (w - row * rw) * 32 + (q & 31);
+  };
+  for (int i0 = 0; i0 < n; i0 += kSeedThreads) {
+    if (threadIdx.x == 0) s_open = 0;
+    __syncthreads();
+    const int i = i0 + (int)threadIdx.x;
+    if (i < n) {
+      const int q = s_queue[i];
+      int u, row;
+      pixel_of(q, u, row);
+      const int seed = seed_ff<ST>(v, f, p, s_T, u, row, __ldg(f.depth + row * f.W + u));
+      if (seed == 1) atomicOr(&s_words[q >> 5], 1u << (q & 31));
+      if (seed == 2) s_last[atomicAdd(&s_open, 1)] = q;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < s_open) {
+      const int q = s_last[threadIdx.x];
+      int u, row;
+      pixel_of(q, u, row);
+      const double r64 = residual_fp64<ST>(v, f, p, T, u, row, __ldg(f.depth + row * f.W + u));
+      if (r64 >= 0.0 && r64 > __dmul_rn(__dmul_rn(p.gamma_d, p.tau_d), p.tau_d))
+        atomicOr(&s_words[q >> 5], 1u << (q & 31));
+    }
+    __syncthreads();  // s_open is reset next
   }
   if (threadIdx.x == 0 && n > 0 && guard_count) atomicAdd(guard_count, (unsigned)n);
   __syncthreads();
