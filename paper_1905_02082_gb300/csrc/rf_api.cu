@@ -474,6 +474,56 @@ __global__ void __launch_bounds__(256) k_batch_out(const BatchStage* __restrict_
   if (blockIdx.x == 0 && threadIdx.x < 16) b.T_out[threadIdx.x] = b.T_dst[32 + threadIdx.x];
 }
 
+// One frame and pose into a volume, and its results back: one launch each
+// (three small copies before and after the replayed graph took 2-3 us apiece).
+struct FrameIn {
+  const uint16_t* depth;
+  const uint8_t* rgb;
+  const double* T;
+  uint16_t* depth_dst;
+  uint8_t* rgb_dst;
+  double* T_dst;
+  size_t npix;
+};
+__global__ void __launch_bounds__(256) k_frame_in(FrameIn a) {
+  const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
+  copy_bytes(a.depth_dst, a.depth, a.npix * 2, tid, nth);
+  copy_bytes(a.rgb_dst, a.rgb, a.npix * 3, tid, nth);
+  if (tid < 16) a.T_dst[tid] = a.T[tid];
+}
+
+struct FrameOut {
+  const double* T;
+  const uint8_t* mask;
+  const rf_track_info* info;  // nullptr: zeros
+  double* T_dst;
+  uint8_t* mask_dst;          // nullable, as info_dst
+  rf_track_info* info_dst;
+  size_t npix;
+};
+__global__ void __launch_bounds__(256) k_frame_out(FrameOut a) {
+  const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
+  if (a.mask_dst) copy_bytes(a.mask_dst, a.mask, a.npix, tid, nth);
+  if (tid < 16) a.T_dst[tid] = a.T[tid];
+  if (tid == 0 && a.info_dst) *a.info_dst = a.info ? *a.info : rf_track_info{};
+}
+
+unsigned copy_ctas(const rf_volume* vol, size_t bytes) {
+  return (unsigned)std::max<size_t>(1, std::min<size_t>((bytes / 16 + 255) / 256, 2 * (size_t)vol->sm_count));
+}
+
+// Whether kernels may read the memory at p: the device's own, or page-locked
+// host memory (which is what rf_frame documents; a pageable pointer goes
+// through the copy engine, as it did).
+bool kernel_readable(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type != cudaMemoryTypeUnregistered && at.devicePointer == p;
+}
+
 rf_status batch_error(rf_batch* b, rf_status s, const std::string& msg) {
   b->last_error = msg;
   return s;
@@ -818,28 +868,20 @@ rf_status rf_process_frame(rf_volume* vol, const rf_frame* frame, const double* 
   cudaGraphExec_t exec = nullptr;
   rf_status s = vol->use_graphs ? frame_graph(vol, frame, first, &exec) : RF_OK;
   if (s) return s;
-  if ((s = check_cuda(vol, cudaMemcpyAsync(vol->d_depth, frame->depth, npix * 2, cudaMemcpyDefault, st),
-                      "depth staging")))
-    return s;
-  if ((s = check_cuda(vol, cudaMemcpyAsync(vol->d_rgb, frame->rgb, npix * 3, cudaMemcpyDefault, st),
-                      "rgb staging")))
-    return s;
-  if ((s = check_cuda(vol, cudaMemcpyAsync(vol->d_T, T_init_dev, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st),
-                      "pose staging")))
-    return s;
-  if ((s = run_frame(vol, frame, first, exec, st))) return s;
-  if ((s = check_cuda(vol, cudaMemcpyAsync(T_out_dev, vol->d_T + 32, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st),
-                      "pose out")))
-    return s;
-  if (mask_dev && (s = check_cuda(vol, cudaMemcpyAsync(mask_dev, vol->d_mask, npix, cudaMemcpyDeviceToDevice, st),
-                                  "mask out")))
-    return s;
-  if (info_dev) {
-    if (first) s = check_cuda(vol, cudaMemsetAsync(info_dev, 0, sizeof(rf_track_info), st), "info out");
-    else s = check_cuda(vol, cudaMemcpyAsync(info_dev, vol->d_info, sizeof(rf_track_info), cudaMemcpyDeviceToDevice, st),
-                        "info out");
-    if (s) return s;
+  FrameIn in = {frame->depth, frame->rgb, T_init_dev, vol->d_depth, vol->d_rgb, vol->d_T, npix};
+  if (!kernel_readable(frame->depth) || !kernel_readable(frame->rgb)) {
+    if ((s = check_cuda(vol, cudaMemcpyAsync(vol->d_depth, frame->depth, npix * 2, cudaMemcpyDefault, st),
+                        "depth staging")) ||
+        (s = check_cuda(vol, cudaMemcpyAsync(vol->d_rgb, frame->rgb, npix * 3, cudaMemcpyDefault, st), "rgb staging")))
+      return s;
+    in.npix = 0;
   }
+  k_frame_in<<<copy_ctas(vol, in.npix * 3), 256, 0, st>>>(in);
+  if ((s = check_cuda(vol, cudaGetLastError(), "frame staging"))) return s;
+  if ((s = run_frame(vol, frame, first, exec, st))) return s;
+  const FrameOut out = {vol->d_T + 32, vol->d_mask, first ? nullptr : vol->d_info, T_out_dev, mask_dev, info_dev, npix};
+  k_frame_out<<<copy_ctas(vol, mask_dev ? npix : 0), 256, 0, st>>>(out);
+  if ((s = check_cuda(vol, cudaGetLastError(), "frame results"))) return s;
   vol->frames++;
   vol->has_model = true;
   return RF_OK;

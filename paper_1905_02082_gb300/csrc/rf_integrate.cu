@@ -14,14 +14,18 @@
 // rounding verified with int64 products after a float guess.
 //
 // Kernels, in stream order:
-//   k_frustum      16x16-tile maximum of valid unmasked depth        (tile/CTA),
-//                  then in its last CTA: quantised pose, counters reset,
-//                  block range of the truncated frustum
+//   k_frustum      16x16-tile maximum of valid unmasked depth       (tile/warp);
+//                  its first CTA quantises the pose and resets the counters,
+//                  its last one takes the block range of the truncated frustum
 //   k_cull         conservative per-block frustum/depth test, warp-aggregated
 //                  append to the candidate list                     (block/thread)
 //   k_integrate    exact per-voxel predicate, lock-free hash insert of blocks
 //                  with updates, read-modify-write of updated voxels (one warp
 //                  per block, persistent grid, static round-robin)
+//   k_nbr_fixup    neighbour tables of the blocks allocated
+// The four are short (3 to 25 us at 640x480), so each may start its CTAs while
+// its predecessor drains (programmatic dependent launch): it reads nothing
+// before griddepcontrol.wait has seen the predecessor complete.
 #include <cmath>
 
 #include "rf_volume.hpp"
@@ -34,24 +38,25 @@ namespace {
 // non-finite pose).
 constexpr long long kMaxSearchBlocks = 1ll << 28;
 
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void start_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Quantised pose (one entry per lane of warp 0: conversions run on the FP64
 // pipe, so they are spread over lanes), the per-frame constants of the voxel
 // loop and the reset of the per-frame counters.
 __device__ __forceinline__ void integ_prep(const double* __restrict__ T, IntegState* st, const int* __restrict__ n_blocks,
-                                           const DevParams& p, int max_um) {
+                                           const DevParams& p) {
   const int a = threadIdx.x;
   if (a < 9) {
     const int i = a / 3, j = a % 3;
     st->A[a] = llround(T[j * 4 + i] * 1073741824.0);  // world -> camera rotation R^T, 2^30 scale
-    st->R[a] = (float)T[i * 4 + j];
+    st->R[a] = (float)T[i * 4 + j];  // (also read by k_cull)
   } else if (a < 12) {
     st->tq[a - 9] = llround(T[(a - 9) * 4 + 3] * 1e6);
     st->t[a - 9] = (float)T[(a - 9) * 4 + 3];
   } else if (a == 12) {
-    st->max_um = max_um;
     st->n_cand = 0;
     st->work = 0;
-    st->clipped = 0;
     st->new_blocks = 0;
     st->updated = 0ull;
     st->pool_before = *n_blocks;
@@ -65,20 +70,22 @@ __device__ __forceinline__ void integ_prep(const double* __restrict__ T, IntegSt
 // Block range of the truncated frustum z in (z_near, zfar], zfar =
 // min(max valid depth + tau, d_max), over the pixel rectangle.  Float math on
 // 8 lanes of one warp (one frustum corner each); the 2-voxel margin covers
-// its rounding.  R, t: the pose as floats (already in st).
-__device__ __forceinline__ void integ_aabb(const DevFrame& f, const DevParams& p, IntegState* st, int max_um,
-                                           int lane) {
+// its rounding.  R, t: the pose as floats.
+__device__ __forceinline__ void integ_aabb(const DevFrame& f, const DevParams& p, const float* R, const float* t,
+                                           IntegState* st, int max_um, int lane) {
+  if (lane == 0) st->max_um = max_um;
   if (max_um < 0) {
     if (lane == 0) {
       st->total = 0;
       st->zfar = 0.0f;
+      st->clipped = 0;
     }
     return;
   }
   const float zfar = fminf((float)max_um * 1e-6f + p.tau, (float)p.dmax_um * 1e-6f);
   bool finite = true;
-  for (int i = 0; i < 9; ++i) finite &= isfinite(st->R[i]) != 0;
-  for (int i = 0; i < 3; ++i) finite &= isfinite(st->t[i]) != 0;
+  for (int i = 0; i < 9; ++i) finite &= isfinite(R[i]) != 0;
+  for (int i = 0; i < 3; ++i) finite &= isfinite(t[i]) != 0;
   float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
   if (lane < 8) {
     const float z = (lane & 4) ? zfar : p.z_near;
@@ -86,7 +93,7 @@ __device__ __forceinline__ void integ_aabb(const DevFrame& f, const DevParams& p
     const float x = (u - f.cx) * f.ifx * z, y = (v - f.cy) * f.ify * z;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const float w = st->R[i * 3] * x + st->R[i * 3 + 1] * y + st->R[i * 3 + 2] * z + st->t[i];
+      const float w = R[i * 3] * x + R[i * 3 + 1] * y + R[i * 3 + 2] * z + t[i];
       lo[i] = w;
       hi[i] = w;
     }
@@ -123,39 +130,69 @@ __device__ __forceinline__ void integ_aabb(const DevFrame& f, const DevParams& p
   st->clipped = clipped ? 1 : 0;  // blocks beyond the key range cannot be stored (reported by k_cull)
 }
 
-// Frustum search, first kernel of an integration.  Per 16x16 tile: the
+// Frustum search, first kernel of an integration.  Per 16x16 tile (a warp
+// each, a lane half a row): the
 // largest valid unmasked depth, and the frame's depth with invalid and masked
 // pixels zeroed (the per-voxel loop then tests one value per pixel).  The
-// last CTA to finish (a ticket counter it resets) then takes the maximum over
-// the tiles and writes the quantised pose, the per-frame constants, the reset
-// counters and the block range of the truncated frustum.
-__global__ void __launch_bounds__(256) k_frustum(DevFrame f, DevParams p, const uint8_t* __restrict__ mask,
-                                                 int* __restrict__ tilemax, IntegState* st, int tiles_x, int ntiles,
-                                                 uint16_t* __restrict__ dm, const double* __restrict__ T,
-                                                 const int* __restrict__ n_blocks) {
+// first CTA meanwhile writes the quantised pose, the per-frame constants and
+// the reset counters (FP64 conversions, a chain of ~2,000 cycles); the
+// last CTA to finish (a ticket counter it resets) takes the maximum over
+// the tiles and writes the block range of the truncated frustum.  Bound by
+// launch and this tail: one wave of 150 CTAs at 640x480 (1,200 CTAs of a tile
+// each, with all of the tail's work in the last one, took 9 us).
+// vec: rows of 8 pixels can be read and written with 16-byte accesses.
+constexpr int kTilesPerCta = 8;
+
+__global__ void __launch_bounds__(32 * kTilesPerCta) k_frustum(DevFrame f, DevParams p, const uint8_t* __restrict__ mask,
+                                                               int* __restrict__ tilemax, IntegState* st, int tiles_x,
+                                                               int ntiles, uint16_t* __restrict__ dm,
+                                                               const double* __restrict__ T,
+                                                               const int* __restrict__ n_blocks, int vec) {
+  wait_for_predecessor();
+  start_successor();
   if (gated_off(f.gate, kModeFirst)) return;
-  const int tile = blockIdx.x;
-  const int u = (tile % tiles_x) * kTile + (threadIdx.x % kTile);
-  const int v = (tile / tiles_x) * kTile + (threadIdx.x / kTile);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = blockIdx.x * kTilesPerCta + warp;
   int d = -1;
-  if (u < f.W && v < f.H) {
-    const int idx = v * f.W + u;
-    const unsigned raw = f.depth[idx];
-    const bool use = pixel_valid(p, raw) && !(mask && mask[idx]);
-    if (use) d = (int)(raw * p.du_um);
-    dm[idx] = use ? (uint16_t)raw : (uint16_t)0;
+  if (tile < ntiles) {
+    const int u = (tile % tiles_x) * kTile + (lane & 1) * 8, v = (tile / tiles_x) * kTile + (lane >> 1);
+    if (v < f.H && u < f.W) {
+      const size_t idx = (size_t)v * f.W + u;
+      if (vec) {  // (then f.W is a multiple of 8: all 8 pixels are in the row)
+        uint4 q = *reinterpret_cast<const uint4*>(f.depth + idx);
+        const uint2 m = mask ? *reinterpret_cast<const uint2*>(mask + idx) : make_uint2(0u, 0u);
+        unsigned w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const unsigned mk = (k < 2 ? m.x : m.y) >> (16 * (k & 1));
+          const unsigned lo = w[k] & 0xFFFFu, hi = w[k] >> 16;
+          const bool ul = pixel_valid(p, lo) && !(mk & 0xFFu), uh = pixel_valid(p, hi) && !(mk & 0xFF00u);
+          if (ul) d = max(d, (int)(lo * p.du_um));
+          if (uh) d = max(d, (int)(hi * p.du_um));
+          w[k] = (ul ? lo : 0u) | ((uh ? hi : 0u) << 16);
+        }
+        *reinterpret_cast<uint4*>(dm + idx) = make_uint4(w[0], w[1], w[2], w[3]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (u + k >= f.W) break;
+          const unsigned raw = f.depth[idx + k];
+          const bool use = pixel_valid(p, raw) && !(mask && mask[idx + k]);
+          if (use) d = max(d, (int)(raw * p.du_um));
+          dm[idx + k] = use ? (uint16_t)raw : (uint16_t)0;
+        }
+      }
+    }
+    d = __reduce_max_sync(0xffffffffu, d);
+    if (lane == 0) tilemax[tile] = d;
   }
-  d = __reduce_max_sync(0xffffffffu, d);
-  __shared__ int s[8];
+  if (blockIdx.x == 0 && threadIdx.x < 32) integ_prep(T, st, n_blocks, p);
+  __shared__ int s[kTilesPerCta];
   __shared__ int s_last;
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = d;
   __syncthreads();
   if (threadIdx.x == 0) {
-    int m = s[0];
-    for (int w = 1; w < 8; ++w) m = max(m, s[w]);
-    tilemax[tile] = m;
-    __threadfence();  // the tile maximum before the ticket
-    s_last = atomicAdd(&st->ticket, 1u) == (unsigned)ntiles - 1u;
+    __threadfence();  // the CTA's tile maxima before the ticket
+    s_last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1u;
   }
   __syncthreads();
   if (!s_last) return;
@@ -163,15 +200,20 @@ __global__ void __launch_bounds__(256) k_frustum(DevFrame f, DevParams p, const 
   int m = -1;
   for (int t = threadIdx.x; t < ntiles; t += blockDim.x) m = max(m, __ldcg(tilemax + t));
   m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) s[warp] = m;
   __syncthreads();
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
-  __syncthreads();
-  int max_um = s[0];
-  for (int w = 1; w < 8; ++w) max_um = max(max_um, s[w]);
-  if (threadIdx.x < 32) integ_prep(T, st, n_blocks, p, max_um);
   if (threadIdx.x == 0) st->ticket = 0u;
-  __syncthreads();  // R and t in st are visible to the whole CTA
-  if (threadIdx.x >= 32 && threadIdx.x < 64) integ_aabb(f, p, st, max_um, threadIdx.x - 32);
+  if (threadIdx.x < 32) {
+    int max_um = s[0];
+#pragma unroll
+    for (int w = 1; w < kTilesPerCta; ++w) max_um = max(max_um, s[w]);
+    float R[9], t[3];  // written by the first CTA before its ticket
+#pragma unroll
+    for (int i = 0; i < 9; ++i) R[i] = __ldcg(&st->R[i]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t[i] = __ldcg(&st->t[i]);
+    integ_aabb(f, p, R, t, st, max_um, lane);
+  }
 }
 
 // Conservative test: may keep blocks without updated voxels, never drops one.
@@ -226,24 +268,29 @@ __device__ bool cull_keep(int bx, int by, int bz, const DevFrame& f, const DevPa
 __global__ void __launch_bounds__(256) k_cull(DevFrame f, DevParams p, IntegState* st, const int* __restrict__ tilemax,
                                               int tiles_x, int tiles_y, int4* __restrict__ cand, long long max_cand,
                                               unsigned* status) {
+  wait_for_predecessor();
+  start_successor();
   if (gated_off(f.gate, kModeFirst)) return;
+  static_assert(sizeof(IntegState) % 4 == 0 && sizeof(IntegState) / 4 <= 256, "copied one word per thread");
   __shared__ IntegState s;
-  if (threadIdx.x == 0) s = *st;
+  if (threadIdx.x < sizeof(IntegState) / 4)
+    reinterpret_cast<unsigned*>(&s)[threadIdx.x] = reinterpret_cast<const unsigned*>(st)[threadIdx.x];
   __syncthreads();
   const int max_um = s.max_um;
   if (s.clipped && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, ST_OUT_OF_RANGE);
-  const long long total = s.total;
-  const long long stride = (long long)gridDim.x * blockDim.x;
+  // (the region has at most kMaxSearchBlocks blocks, and the grid fewer threads: 32-bit indices)
+  const unsigned total = (unsigned)s.total, stride = gridDim.x * blockDim.x;
+  const unsigned dx = (unsigned)s.dims[0], dy = (unsigned)s.dims[1];
   const int lane = threadIdx.x & 31;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < total; base += stride) {
-    const long long idx = base + threadIdx.x;
+  for (unsigned base = blockIdx.x * blockDim.x; base < total; base += stride) {
+    const unsigned idx = base + threadIdx.x;
     bool keep = false;
     int bx = 0, by = 0, bz = 0;
     if (idx < total) {
-      const long long dx = s.dims[0], dy = s.dims[1];
-      bx = s.bmin[0] + (int)(idx % dx);
-      by = s.bmin[1] + (int)((idx / dx) % dy);
-      bz = s.bmin[2] + (int)(idx / (dx * dy));
+      const unsigned row = idx / dx, slice = row / dy;
+      bx = s.bmin[0] + (int)(idx - row * dx);
+      by = s.bmin[1] + (int)(row - slice * dy);
+      bz = s.bmin[2] + (int)slice;
       keep = cull_keep(bx, by, bz, f, p, s, tilemax, tiles_x, tiles_y, max_um);
     }
     const unsigned ballot = __ballot_sync(0xffffffffu, keep);
@@ -704,6 +751,8 @@ __global__ void __launch_bounds__(kIntegThreads, 8) k_integrate(DevVol v, DevFra
   __shared__ unsigned short s_aq[kIntegWarps][kBV];  // voxels queued for the exact path
   __shared__ LaneConsts s_lc[kIntegThreads];
   __shared__ long long s_S[kIntegWarps][4];
+  wait_for_predecessor();
+  start_successor();
   if (gated_off(f.gate, kModeFirst)) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (threadIdx.x < 9) sh.A[threadIdx.x] = st->A[threadIdx.x];
@@ -756,6 +805,8 @@ __device__ __forceinline__ void fixup_entry(const DevVol& v, int b, int k) {
 
 __global__ void __launch_bounds__(256) k_nbr_fixup(DevVol v, const int* __restrict__ lo_ptr, int lo_value,
                                                    const int* gate) {
+  wait_for_predecessor();
+  start_successor();
   if (gated_off(gate, kModeFirst)) return;
   const int lo = lo_ptr ? *lo_ptr : lo_value;
   const int hi = min(*(volatile int*)v.n_blocks, v.max_blocks);
@@ -766,33 +817,50 @@ __global__ void __launch_bounds__(256) k_nbr_fixup(DevVol v, const int* __restri
 
 }  // namespace
 
-rf_status launch_nbr_fixup(rf_volume* vol, const int* lo_ptr, int lo, cudaStream_t st, const int* gate) {
-  k_nbr_fixup<<<vol->sm_count * vol->launch.fixup_ctas_per_sm, 256, 0, st>>>(vol->dv, lo_ptr, lo, gate);
-  return check_cuda(vol, cudaGetLastError(), "neighbour table launch");
+// A launch that may begin while its predecessor in the stream drains (the
+// kernels above wait for it themselves).
+template <class... P, class... A>
+static rf_status launch_after(rf_volume* vol, void (*kernel)(P...), int grid, int threads, cudaStream_t st,
+                              const char* what, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return check_cuda(vol, cudaLaunchKernelEx(&cfg, kernel, P(args)...), what);
 }
 
-// The frustum search of an integration: prep, tile maxima, AABB, cull.
+rf_status launch_nbr_fixup(rf_volume* vol, const int* lo_ptr, int lo, cudaStream_t st, const int* gate) {
+  return launch_after(vol, k_nbr_fixup, vol->sm_count * vol->launch.fixup_ctas_per_sm, 256, st,
+                      "neighbour table launch", vol->dv, lo_ptr, lo, gate);
+}
+
+// The frustum search of an integration: tile maxima, prep, AABB, cull.
 static rf_status launch_frustum(rf_volume* vol, const DevFrame& f, const double* T, const uint8_t* mask, cudaStream_t st) {
-  const int tiles_x = (f.W + kTile - 1) / kTile, tiles_y = (f.H + kTile - 1) / kTile;
-  k_frustum<<<tiles_x * tiles_y, 256, 0, st>>>(f, vol->dp, mask, vol->d_tilemax, vol->d_integ, tiles_x,
-                                               tiles_x * tiles_y, vol->d_dmask, T, vol->d_nblocks);
-  k_cull<<<vol->sm_count * vol->launch.cull_ctas_per_sm, 256, 0, st>>>(f, vol->dp, vol->d_integ, vol->d_tilemax, tiles_x, tiles_y, vol->d_cand,
-                                            vol->p.max_candidates, vol->d_status);
-  return check_cuda(vol, cudaGetLastError(), "frustum launch");
+  const int tiles_x = (f.W + kTile - 1) / kTile, tiles_y = (f.H + kTile - 1) / kTile, ntiles = tiles_x * tiles_y;
+  const int vec = f.W % 8 == 0 && (reinterpret_cast<uintptr_t>(f.depth) & 15) == 0 &&
+                  (reinterpret_cast<uintptr_t>(mask) & 7) == 0;  // (d_dmask is an allocation of its own: aligned)
+  rf_status s = launch_after(vol, k_frustum, (ntiles + kTilesPerCta - 1) / kTilesPerCta, 32 * kTilesPerCta, st,
+                             "frustum launch", f, vol->dp, mask, vol->d_tilemax, vol->d_integ, tiles_x, ntiles,
+                             vol->d_dmask, T, vol->d_nblocks, vec);
+  if (s != RF_OK) return s;
+  return launch_after(vol, k_cull, vol->sm_count * vol->launch.cull_ctas_per_sm, 256, st, "cull launch", f, vol->dp,
+                      vol->d_integ, vol->d_tilemax, tiles_x, tiles_y, vol->d_cand, (long long)vol->p.max_candidates,
+                      vol->d_status);
 }
 
 rf_status launch_integrate(rf_volume* vol, const DevFrame& f, const double* T, const uint8_t* mask, cudaStream_t st) {
   rf_status s = launch_frustum(vol, f, T, mask, st);
   if (s != RF_OK) return s;
   prof_record(vol, EV_KERNEL0, st);
-  if (vol->p.storage == RF_STORAGE_FP16)
-    k_integrate<RF_STORAGE_FP16><<<vol->sm_count * vol->launch.integrate_ctas_per_sm, kIntegThreads, 0, st>>>(vol->dv, f, vol->dp, vol->d_dmask, vol->d_integ,
-                                                                             vol->d_cand, vol->p.max_candidates);
-  else
-    k_integrate<RF_STORAGE_FP32><<<vol->sm_count * vol->launch.integrate_ctas_per_sm, kIntegThreads, 0, st>>>(vol->dv, f, vol->dp, vol->d_dmask, vol->d_integ,
-                                                                             vol->d_cand, vol->p.max_candidates);
+  s = launch_after(vol, vol->p.storage == RF_STORAGE_FP16 ? k_integrate<RF_STORAGE_FP16> : k_integrate<RF_STORAGE_FP32>,
+                   vol->sm_count * vol->launch.integrate_ctas_per_sm, kIntegThreads, st, "integrate launch", vol->dv, f,
+                   vol->dp, vol->d_dmask, vol->d_integ, vol->d_cand, (long long)vol->p.max_candidates);
   prof_record(vol, EV_KERNEL1, st);
-  s = check_cuda(vol, cudaGetLastError(), "integrate launch");
   if (s != RF_OK) return s;
   return launch_nbr_fixup(vol, &vol->d_integ->pool_before, 0, st, f.gate);
 }
