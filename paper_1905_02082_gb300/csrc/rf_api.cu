@@ -402,14 +402,16 @@ struct rf_batch_graph {
   RegDesc* d_desc = nullptr;   // [2][n]: first and second registration
   FillDesc* d_flood = nullptr;  // [n]: erosion, flood fill, dilation
   MaskDesc* d_mask = nullptr;   // [n]: seeds
-  // [n] BatchStage, then per registration launch (ngroups of them): CTA ->
-  // stream [total], then the n + 1 group starts
+  // [n] BatchStage, then per flood-fill launch (ngroups of them): CTA ->
+  // stream [ff_ctas], then the n + 1 group starts; then the registrations'
+  // queue: CTA -> group [total], group starts [n + 1], streams in order [n],
+  // their number, and per registration pass a counter and [n] group words
   void* d_table = nullptr;
   std::vector<unsigned char> h_table;
   int total_ctas = 0;
-  int ngroups = 1;  // registration launches per registration
-  int gsize = 1;    // tracked streams per launch at most
-  int ff_ctas = 0;  // CTAs of a batched flood-fill launch (its own maps follow the registration's)
+  int ngroups = 1;  // flood-fill launches
+  int gsize = 1;    // tracked streams registered at the same time, and per flood-fill launch, at most
+  int ff_ctas = 0;  // CTAs of a batched flood-fill launch
 };
 
 struct rf_batch {
@@ -552,22 +554,32 @@ void join_aux(rf_batch* b, cudaStream_t cs) {
   }
 }
 
-size_t table_bytes(int n, int total_ctas, int ff_ctas, int ngroups) {
-  return sizeof(BatchStage) * n + sizeof(int) * (size_t)ngroups * ((total_ctas + n + 1) + (ff_ctas + n + 1));
-}
+// Layout of the table after the BatchStage entries, in ints.
+struct BatchTable {
+  int n, total, ff, ngroups;
+  int ff_len() const { return ff + n + 1; }
+  size_t group() const { return (size_t)ngroups * ff_len(); }
+  size_t first() const { return group() + total; }
+  size_t order() const { return first() + n + 1; }
+  size_t length() const { return order() + n; }
+  size_t counter(int pass) const { return length() + 1 + (size_t)pass * (n + 1); }  // then the group words
+  size_t ints() const { return counter(2); }
+};
+BatchTable table_of(const rf_batch_graph& g, int n) { return BatchTable{n, g.total_ctas, g.ff_ctas, g.ngroups}; }
 
 // Captures the batch graph for one shape.  Every stream gets the full path;
 // which streams actually track is decided per replay by the uploaded table.
 rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<double>& sig, rf_batch_graph* out) {
   const int n = (int)b->vols.size();
   out->total_ctas = b->vols[0]->reg_grid;
-  // the tracked streams of a call run in groups of at most gsize per
-  // registration launch (launch setting batch_group; 0: all in one)
+  // at most gsize tracked streams of a call are registered at the same time
+  // (launch setting batch_group; 0: all)
   const int bg = b->vols[0]->launch.batch_group;
   out->gsize = bg > 0 ? std::min(bg, n) : n;
   out->ngroups = (n + out->gsize - 1) / out->gsize;
   out->ff_ctas = b->vols[0]->ff_grid;
-  out->h_table.assign(table_bytes(n, out->total_ctas, out->ff_ctas, out->ngroups), 0);
+  const BatchTable bt = table_of(*out, n);
+  out->h_table.assign(sizeof(BatchStage) * n + sizeof(int) * bt.ints(), 0);
   cudaError_t e = cudaMalloc(&out->d_table, out->h_table.size());
   if (e != cudaSuccess) return batch_error(b, RF_ERR_CUDA, std::string("batch table: ") + cudaGetErrorString(e));
   const void* out_table = out->d_table;
@@ -611,10 +623,13 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     s = batch_error(b, RF_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e));
   } else {
     const BatchStage* table = static_cast<const BatchStage*>(out->d_table);
-    const int* maps = reinterpret_cast<const int*>(table + n);
-    const int map_len = out->total_ctas + n + 1;
-    const int* ff_maps = maps + out->ngroups * map_len;
-    const int ff_len = out->ff_ctas + n + 1;
+    int* words = reinterpret_cast<int*>(static_cast<BatchStage*>(out->d_table) + n);
+    const int* ff_maps = words;
+    const int ff_len = bt.ff_len();
+    auto queue = [&](int pass) {
+      unsigned* c = reinterpret_cast<unsigned*>(words + bt.counter(pass));
+      return RegQueue{words + bt.group(), words + bt.first(), words + bt.order(), c + 1, c, words + bt.length()};
+    };
     int max_npix = 1, max_seed_blocks = 1;
     for (int i = 0; i < n; ++i) {
       max_npix = std::max(max_npix, f[i].H * f[i].W);
@@ -622,9 +637,7 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     }
     const dim3 copy_grid((unsigned)std::min((max_npix * 3 / 16 + 255) / 256, 64), (unsigned)n);
     k_batch_stage<<<copy_grid, 256, 0, cs>>>(table);
-    for (int gi = 0; gi < out->ngroups && !s; ++gi)
-      s = launch_register_batch(b->vols[0], out->d_desc, maps + gi * map_len, maps + gi * map_len + out->total_ctas,
-                                out->total_ctas, cs);
+    s = launch_register_batch(b->vols[0], out->d_desc, queue(0), out->total_ctas, cs);
     // residual seeds of every stream: one launch (the mask words were reset by
     // the staging kernel); erosion, flood fill and dilation: one cooperative
     // launch per group of streams
@@ -632,9 +645,7 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     for (int gi = 0; gi < out->ngroups && !s; ++gi)
       s = launch_fill_batch(b->vols[0], out->d_flood, ff_maps + gi * ff_len, ff_maps + gi * ff_len + out->ff_ctas,
                             out->ff_ctas, cs);
-    for (int gi = 0; gi < out->ngroups && !s; ++gi)
-      s = launch_register_batch(b->vols[0], out->d_desc + n, maps + gi * map_len,
-                                maps + gi * map_len + out->total_ctas, out->total_ctas, cs);
+    if (!s) s = launch_register_batch(b->vols[0], out->d_desc + n, queue(1), out->total_ctas, cs);
     // integrations: concurrent (one launch over all streams' candidate
     // blocks is no faster: the per-voxel update is latency-bound at its
     // occupancy, and concurrent launches overlap the streams' frustum searches)
@@ -1267,10 +1278,8 @@ rf_status rf_batch_process(rf_batch* b, const rf_frame* frames, const double* co
   }
   // per-call table: staging pointers and modes, then the registration CTA map
   BatchStage* tab = reinterpret_cast<BatchStage*>(g->h_table.data());
-  int* maps = reinterpret_cast<int*>(tab + n);
-  const int map_len = g->total_ctas + n + 1;
-  int* ff_maps = maps + g->ngroups * map_len;
-  const int ff_len = g->ff_ctas + n + 1;
+  const BatchTable bt = table_of(*g, n);
+  int* words = reinterpret_cast<int*>(tab + n);
   std::vector<int> tracked;
   for (int i = 0; i < n; ++i) {
     rf_volume* v = b->vols[i];
@@ -1289,15 +1298,30 @@ rf_status rf_batch_process(rf_batch* b, const rf_frame* frames, const double* co
     t.mode = mode[i];
     if (mode[i] == kModeTrack) tracked.push_back(i);
   }
-  // registration launch gi takes the tracked streams gi*gsize .. gi*gsize+gsize-1
+  // flood-fill launch gi takes the tracked streams gi*gsize .. gi*gsize+gsize-1
   // (in stream order), CTAs split among them by pixel count
-  // (the flood fills use the same groups, with maps over their own CTA count)
   for (int gi = 0; gi < g->ngroups; ++gi) {
     std::vector<double> w(n, 0.0);
     for (int k = gi * g->gsize; k < std::min((int)tracked.size(), (gi + 1) * g->gsize); ++k)
       w[tracked[k]] = (double)tab[tracked[k]].npix;
-    fill_cta_map(w, g->total_ctas, maps + gi * map_len);
-    fill_cta_map(w, g->ff_ctas, ff_maps + gi * ff_len);
+    fill_cta_map(w, g->ff_ctas, words + gi * bt.ff_len());
+  }
+  // registrations: the tracked streams in a queue, the largest first; one
+  // group of CTAs for each while there are at most gsize of them (sized by
+  // pixel count), else gsize equal groups that take the next when done
+  std::vector<int> order = tracked;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return tab[a].npix > tab[c].npix; });
+  const int reg_groups = std::min((int)order.size(), g->gsize);
+  {
+    std::vector<double> w(n, 0.0);
+    for (int k = 0; k < reg_groups; ++k) w[k] = (int)order.size() <= g->gsize ? (double)tab[order[k]].npix : 1.0;
+    fill_cta_map(w, g->total_ctas, words + bt.group());
+  }
+  std::copy(order.begin(), order.end(), words + bt.order());
+  words[bt.length()] = (int)order.size();
+  for (int pass = 0; pass < 2; ++pass) {
+    words[bt.counter(pass)] = reg_groups;
+    std::fill_n(words + bt.counter(pass) + 1, n, 0);
   }
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(g->d_table, g->h_table.data(), g->h_table.size(), cudaMemcpyHostToDevice, st);

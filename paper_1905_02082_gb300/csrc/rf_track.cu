@@ -487,6 +487,11 @@ __device__ __noinline__ bool lm_candidate(const float* sums, const float* hi, co
 
 constexpr int kRegThreads = 512;
 constexpr int kRegWarps = kRegThreads / 32;
+// Steps (a chunk per slot each) between CTA barriers in a batch, where a CTA
+// has several chunks: the warps of a CTA need not keep step with its slowest
+// one at each.  A warp per chunk then sums the warps' partials (at most 4 slots
+// x 4 steps).
+constexpr int kBatchSteps = 4;
 
 // Pixels per partial sum: a fixed chunk of the sampled pixels of a level, a
 // function of their number only, so the partials, and thus the result, do not
@@ -587,10 +592,10 @@ __device__ __forceinline__ void leave_registration(const RegDesc& d, int G, unsi
 // the next candidate of an acceptance while another warp decides which of the
 // two applies.  The first of them shares warp 0's scheduler and so leaves its
 // instruction cache holding the step's code.
-template <int ST>
-__device__ void register_body(const RegDesc& d, int lb, int G) {
+template <int ST, int kStepsPerBarrier>
+__device__ __forceinline__ void register_body(const RegDesc& d, int lb, int G) {
   __shared__ RegShared S;
-  __shared__ float red[2][kRegWarps][32];  // per-warp sums of a chunk, double-buffered by step parity
+  __shared__ float red[2][kStepsPerBarrier][kRegWarps][32];  // per-warp sums of chunks, double-buffered
   constexpr int kRejectWarp = 12, kDecideWarp = 13;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const DevFrame& f = d.f;
@@ -696,61 +701,69 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
       const float4* pose = S.pose[first ? iT : iC];
       ulonglong2* part = d.partials + (size_t)(eval & 1u) * kRegWords * d.max_slots;
       const unsigned tag = tag0 + eval + 1u;
-      for (int step = 0; lb + G * slots * step < nchunks; ++step) {
-        const int ch = lb + G * (slot + slots * step);
-        int end;
-        int i = bounds(ch, end);
-        const bool any = __any_sync(0xffffffffu, i < end);
+      int par = 0;
+      for (int step0 = 0; lb + G * slots * step0 < nchunks; step0 += kStepsPerBarrier) {
+        for (int sb = 0; sb < kStepsPerBarrier && lb + G * slots * (step0 + sb) < nchunks; ++sb) {
+          const int ch = lb + G * (slot + slots * (step0 + sb));
+          int end;
+          int i = bounds(ch, end);
+          const bool any = __any_sync(0xffffffffu, i < end);
 #pragma unroll 1
-        while (i < end) {
-          const float4 r = rec;
-          const unsigned long long cj = cached;
-          const int here = i;
-          i += width;
-          if (i < end) fetch(i);  // the next sample's record
-          if (r.z > 0.0f) {
-            const unsigned long long fresh = add_sample<ST>(d.v, c, pose, r.x, r.y, r.z, r.w, cj, acc);
-            if (fresh != kEmpty) d.pxcache[pixel_of_sample(L, f.W, here)] = fresh;
-          }
-        }
-        // chunk partial: a butterfly over the warp that halves the vector at
-        // every step (31 shuffles for 32 slots) and leaves component c on
-        // lane c, then the warps in fixed order
-        float* mine = &red[step & 1][warp][lane];
-        if (any) {
-          __syncwarp();
-          float v[32];
-#pragma unroll
-          for (int q = 0; q < 28; ++q) {
-            float a, b;
-            unpk(acc.v[q], a, b);
-            v[q] = a + b;
-          }
-          v[28] = acc.n;
-          v[29] = v[30] = v[31] = 0.0f;
-#pragma unroll
-          for (int h = 16; h > 0; h >>= 1) {
-            const bool upper = (lane & h) != 0;
-#pragma unroll
-            for (int q = 0; q < h; ++q) {
-              const float keep = upper ? v[q + h] : v[q];
-              const float send = upper ? v[q] : v[q + h];
-              v[q] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+          while (i < end) {
+            const float4 r = rec;
+            const unsigned long long cj = cached;
+            const int here = i;
+            i += width;
+            if (i < end) fetch(i);  // the next sample's record
+            if (r.z > 0.0f) {
+              const unsigned long long fresh = add_sample<ST>(d.v, c, pose, r.x, r.y, r.z, r.w, cj, acc);
+              if (fresh != kEmpty) d.pxcache[pixel_of_sample(L, f.W, here)] = fresh;
             }
           }
-          *mine = v[0];
-        } else {
-          *mine = 0.0f;
+          // chunk partial: a butterfly over the warp that halves the vector at
+          // every step (31 shuffles for 32 slots) and leaves component c on
+          // lane c, then the warps in fixed order
+          float* mine = &red[par][sb][warp][lane];
+          if (any) {
+            __syncwarp();
+            float v[32];
+#pragma unroll
+            for (int q = 0; q < 28; ++q) {
+              float a, b;
+              unpk(acc.v[q], a, b);
+              v[q] = a + b;
+            }
+            v[28] = acc.n;
+            v[29] = v[30] = v[31] = 0.0f;
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) {
+              const bool upper = (lane & h) != 0;
+#pragma unroll
+              for (int q = 0; q < h; ++q) {
+                const float keep = upper ? v[q + h] : v[q];
+                const float send = upper ? v[q] : v[q + h];
+                v[q] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+              }
+            }
+            *mine = v[0];
+          } else {
+            *mine = 0.0f;
+          }
+          clear(acc);
+          if (lb + G * slots * (step0 + sb + 1) < nchunks) {  // (the last step's follows below, after its partial)
+            const int j = bounds(ch + G * slots, end);
+            if (j < end) fetch(j);
+          }
         }
         __syncthreads();
-        // the chunk partial of each slot: its warps' sums in order; lane w < 10
+        // the chunk partials: the warps' sums of each in order; lane w < 10
         // writes components 3 w .. 3 w + 2 with the tag.  No barrier after
-        // it: the next step writes the other buffer, and this one again only
-        // after the next step's barrier, which these reads precede.
-        const int cs = lb + G * (warp + slots * step);
-        if (warp < slots && cs < nchunks) {
+        // it: the next steps write the other buffer, and this one again only
+        // after their barrier, which these reads precede.
+        const int sb = warp / slots, cs = lb + G * (warp - sb * slots + slots * (step0 + sb));
+        if (sb < kStepsPerBarrier && cs < nchunks) {
           const int wpc = width / 32;
-          const float* from = &red[step & 1][warp * wpc][lane];
+          const float* from = &red[par][sb][(warp - sb * slots) * wpc][lane];
           float t[kRegWarps], sv = 0.0f;
 #pragma unroll
           for (int w = 0; w < kRegWarps; ++w) t[w] = w < wpc ? from[32 * w] : 0.0f;
@@ -761,14 +774,16 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
           const unsigned s2 = __float_as_uint(__shfl_sync(0xffffffffu, sv, (3 * lane + 2) & 31));
           if (lane < kRegWords) st_relaxed_gpu_b128(part + lane * d.max_slots + cs, s0, s1, s2, tag);
         }
-        const bool more = lb + G * slots * (step + 1) < nchunks;
+        par ^= 1;
+      }
+      if (lb < nchunks) {
         // arrival: one relaxed count per CTA (other warps' partial stores may
         // still be on their way: the readers check the tags)
-        if (!more && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
-        // for the next step (or the next evaluation, which samples the same
-        // pixels), during the exchange: empty sums and the first record
-        clear(acc);
-        const int j = bounds(more ? ch + G * slots : lb + G * slot, end);
+        if (threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
+        // for the next evaluation, which samples the same pixels, during the
+        // exchange: the first record
+        int end;
+        const int j = bounds(lb + G * slot, end);
         if (j < end) fetch(j);
       }
       if (lb >= nchunks && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
@@ -903,23 +918,67 @@ __device__ void register_body(const RegDesc& d, int lb, int G) {
 
 // One registration on the whole grid.
 template <int ST>
-__global__ void __launch_bounds__(kRegThreads, 1) k_register(RegDesc d) { register_body<ST>(d, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(kRegThreads, 1) k_register(RegDesc d) {
+  register_body<ST, 1>(d, blockIdx.x, gridDim.x);
+}
 
-// Several independent registrations in one cooperative launch: CTA b runs
-// stream cta_stream[b] as member b - first[s] of a group of first[s+1] -
-// first[s] CTAs.  Groups never wait on each other.  A CTA mapped to stream
-// -1 has no work (streams that sit a batch out, or are on their first frame,
-// get no CTAs; the map is rewritten per batch without re-capturing the graph).
+// The registrations of a batch in one cooperative launch.  CTA b is member
+// b - first[g] of group g = cta_group[b] (-1: no work) of first[g + 1] -
+// first[g] CTAs; groups never wait on each other.  A group registers the
+// streams of the queue one after the other: its first is order[g], its leader
+// takes the next from the shared counter and tells the group's other CTAs
+// through next[g] (round in the upper half, queue position + 1 in the lower).
+// Streams need 12 to 23 evaluations and have up to 12 times the pixels of
+// others; with a fixed set of streams per launch a quarter of the SMs' time was
+// spent waiting for the launch's last stream.  The queue and its counters
+// are part of the table that each call uploads.
 template <int ST>
 __global__ void __launch_bounds__(kRegThreads, 1)
-    k_register_batch(const RegDesc* __restrict__ descs, const int* __restrict__ cta_stream,
-                     const int* __restrict__ first) {
+    k_register_batch(const RegDesc* __restrict__ descs, const int* __restrict__ cta_group, const int* __restrict__ first,
+                     const int* __restrict__ order, unsigned* next, unsigned* counter, const int* __restrict__ length) {
   __shared__ RegDesc sd;
-  const int s = cta_stream[blockIdx.x];
-  if (s < 0) return;
-  if (threadIdx.x == 0) sd = descs[s];
-  __syncthreads();
-  register_body<ST>(sd, blockIdx.x - first[s], first[s + 1] - first[s]);
+  __shared__ int s_at;
+  const int g = cta_group[blockIdx.x];
+  if (g < 0) return;
+  const int lb = blockIdx.x - first[g], G = first[g + 1] - first[g], n = *length;
+  for (unsigned round = 0;; ++round) {
+    if (threadIdx.x == 0) {
+      int at = g;
+      if (round > 0) {
+        if (lb == 0) {
+          at = (int)atomicAdd(counter, 1u);
+          at = min(at, n);
+          st_relaxed_gpu_u32(next + g, (round << 16) | (unsigned)(at + 1));
+        } else {
+          // every member of the last registration has taken part in it, so it
+          // has read its round's word
+          unsigned w = 0u;
+          long long spins = 0;
+          for (;;) {
+            w = ld_relaxed_gpu(next + g);
+            if ((w >> 16) == round) break;
+            if (++spins > sd.spin_limit) {
+              atomicOr(sd.status, ST_BARRIER);
+              w = (unsigned)n + 1u;
+              break;
+            }
+            if (spins > 4096) __nanosleep(64);
+          }
+          at = (int)(w & 0xFFFFu) - 1;
+        }
+      }
+      s_at = at;
+    }
+    __syncthreads();
+    if (s_at >= n) return;
+    const RegDesc* from = descs + order[s_at];
+    static_assert(sizeof(RegDesc) % 4 == 0, "copied in words");
+    for (unsigned i = threadIdx.x; i < sizeof(RegDesc) / 4; i += kRegThreads)
+      reinterpret_cast<unsigned*>(&sd)[i] = reinterpret_cast<const unsigned*>(from)[i];
+    __syncthreads();
+    register_body<ST, kBatchSteps>(sd, lb, G);
+    __syncthreads();
+  }
 }
 
 }  // namespace
@@ -1000,9 +1059,11 @@ rf_status launch_track(rf_volume* vol, const DevFrame& f, const double* T_init, 
   return launch_coop(vol, fn, std::min(vol->reg_grid, most), args, st);
 }
 
-rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const int* cta_stream, const int* first,
-                                int total_ctas, cudaStream_t st) {
-  void* args[] = {(void*)&descs, (void*)&cta_stream, (void*)&first};
+rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const RegQueue& q, int total_ctas,
+                                cudaStream_t st) {
+  RegQueue a = q;
+  void* args[] = {(void*)&descs, (void*)&a.cta_group, (void*)&a.first, (void*)&a.order,
+                  (void*)&a.next, (void*)&a.counter, (void*)&a.length};
   const void* fn = vol->p.storage == RF_STORAGE_FP16 ? (const void*)k_register_batch<RF_STORAGE_FP16>
                                                      : (const void*)k_register_batch<RF_STORAGE_FP32>;
   return launch_coop(vol, fn, total_ctas, args, st);
