@@ -256,8 +256,17 @@ __device__ bool cull_keep(int bx, int by, int bz, const DevFrame& f, const DevPa
   const int tx0 = u0 / kTile, tx1 = u1 / kTile, ty0 = v0 / kTile, ty1 = v1 / kTile;
   int m = -1;
   if ((tx1 - tx0 + 1) * (ty1 - ty0 + 1) <= 64) {
-    for (int ty = ty0; ty <= ty1; ++ty)
-      for (int tx = tx0; tx <= tx1; ++tx) m = max(m, __ldg(tilemax + ty * tiles_x + tx));
+    // 16 tiles at a time, their loads issued together (beyond the range: its
+    // last row or column again): one load after the other was most of k_cull
+    for (int ty = ty0; ty <= ty1; ty += 4)
+      for (int tx = tx0; tx <= tx1; tx += 4) {
+        int q[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          q[k] = __ldg(tilemax + min(ty + (k >> 2), ty1) * tiles_x + min(tx + (k & 3), tx1));
+#pragma unroll
+        for (int k = 0; k < 16; ++k) m = max(m, q[k]);
+      }
   } else {
     m = max_um;
   }
