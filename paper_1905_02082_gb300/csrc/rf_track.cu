@@ -116,9 +116,9 @@ __device__ __forceinline__ unsigned long long add_sample(const DevVol& v, const 
                                                          float x, float y, float z, float off,
                                                          unsigned long long cached, Acc& acc) {
   const float4 r0 = pose[0], r1 = pose[1], r2 = pose[2];
-  const float px = fmaf(r0.z, z, fmaf(r0.y, y, r0.x * x)) + r0.w;
-  const float py = fmaf(r1.z, z, fmaf(r1.y, y, r1.x * x)) + r1.w;
-  const float pz = fmaf(r2.z, z, fmaf(r2.y, y, r2.x * x)) + r2.w;
+  const float px = fmaf(r0.z, z, fmaf(r0.y, y, fmaf(r0.x, x, r0.w)));
+  const float py = fmaf(r1.z, z, fmaf(r1.y, y, fmaf(r1.x, x, r1.w)));
+  const float pz = fmaf(r2.z, z, fmaf(r2.y, y, fmaf(r2.x, x, r2.w)));
   const float qx = px * c.inv_voxel, qy = py * c.inv_voxel, qz = pz * c.inv_voxel;
   // floor: adding 1.5 * 2^23 rounded down leaves the integer in the low
   // mantissa bits (exact for |q| < 2^22)
