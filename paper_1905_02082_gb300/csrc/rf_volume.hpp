@@ -35,8 +35,8 @@ struct rf_volume {
   // registration scratch
   // 2 x kRegWords x max_slots tagged partial sums of the registration (three
   // floats, then the tag in the top 32 bits of each 16-byte word).  Mesh
-  // extraction and virtual-depth filling reuse the first 8 bytes as a counter
-  // between registrations: they are below the first word's tag.
+  // extraction reuses the first 8 bytes as a counter between registrations:
+  // they are below the first word's tag.
   ulonglong2* d_partials = nullptr;
   int max_slots = 0;
   unsigned* d_regtags = nullptr;  // registration tag base and leaving count
