@@ -335,9 +335,11 @@ rf_status rf_set_launch_config(rf_volume* vol, const rf_launch_config* cfg);
 /* Bounded waits (a property of the library; the paper has no counterpart).
  * Every grid-wide wait of the cooperative kernels (the flood fill's grid
  * barrier; the registration's wait for every CTA's partial sums of a cost
- * evaluation) polls at most spin_limit times before it gives up: the kernel
- * then records RF_ERR_NOT_CONVERGED in the status word (rf_sync_status) and
- * returns, and the volume stays usable.  spin_limit 0 restores the default,
+ * evaluation; in a batch a CTA's wait for its group's next stream) polls at
+ * most spin_limit times before it gives up: the kernel then records
+ * RF_ERR_NOT_CONVERGED in the status word (rf_sync_status; in a batch: of every
+ * stream whose registration did not run or finish) and returns, and the
+ * volumes stay usable.  spin_limit 0 restores the default,
  * 2^24 polls (about one second).  extra_arrivals is fault injection for
  * tests: with extra_arrivals > 0 each wait expects that many arrivals beyond
  * the CTAs launched, which never come, so every wait runs out and the error

@@ -12,6 +12,7 @@
 
 #include "rf_cta_map.hpp"
 #include "rf_half.hpp"
+#include "rf_queue.hpp"
 #include "rf_volume.hpp"
 
 namespace rf {
@@ -405,7 +406,7 @@ struct rf_batch_graph {
   // [n] BatchStage, then per flood-fill launch (ngroups of them): CTA ->
   // stream [ff_ctas], then the n + 1 group starts; then the registrations'
   // queue: CTA -> group [total], group starts [n + 1], streams in order [n],
-  // their number, and per registration pass a counter and [n] group words
+  // their number, and per registration pass two counters and [n] links
   void* d_table = nullptr;
   std::vector<unsigned char> h_table;
   int total_ctas = 0;
@@ -562,7 +563,7 @@ struct BatchTable {
   size_t first() const { return group() + total; }
   size_t order() const { return first() + n + 1; }
   size_t length() const { return order() + n; }
-  size_t counter(int pass) const { return length() + 1 + (size_t)pass * (n + 1); }  // then the group words
+  size_t counter(int pass) const { return length() + 1 + (size_t)pass * (n + 2); }  // then the groups left and the links
   size_t ints() const { return counter(2); }
 };
 BatchTable table_of(const rf_batch_graph& g, int n) { return BatchTable{n, g.total_ctas, g.ff_ctas, g.ngroups}; }
@@ -628,7 +629,7 @@ rf_status batch_capture(rf_batch* b, const rf_frame* frames, const std::vector<d
     const int ff_len = bt.ff_len();
     auto queue = [&](int pass) {
       unsigned* c = reinterpret_cast<unsigned*>(words + bt.counter(pass));
-      return RegQueue{words + bt.group(), words + bt.first(), words + bt.order(), c + 1, c, words + bt.length()};
+      return RegQueue{words + bt.group(), words + bt.first(), words + bt.order(), words + bt.length(), c, c + 1, c + 2};
     };
     int max_npix = 1, max_seed_blocks = 1;
     for (int i = 0; i < n; ++i) {
@@ -793,6 +794,9 @@ rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_bl
   if (!s) s = check_cuda(vol, cudaMemset(vol->d_status, 0, sizeof(unsigned)), "status reset");
   // the frustum search's ticket counter starts at 0
   if (!s) s = check_cuda(vol, cudaMemset(vol->d_integ, 0, sizeof(IntegState)), "integration state reset");
+  // (a frame whose registration did not finish is integrated at the pose that
+  // its buffer holds: a pose of zeros sees no voxel)
+  if (!s) s = check_cuda(vol, cudaMemset(vol->d_T, 0, 48 * sizeof(double)), "pose reset");
   // registration tags start at 0 (base, counts) with every partial-sum word's tag 0
   if (!s) s = check_cuda(vol, cudaMemset(vol->d_regtags, 0, 3 * sizeof(unsigned)), "tag reset");
   if (!s)
@@ -1320,8 +1324,8 @@ rf_status rf_batch_process(rf_batch* b, const rf_frame* frames, const double* co
   std::copy(order.begin(), order.end(), words + bt.order());
   words[bt.length()] = (int)order.size();
   for (int pass = 0; pass < 2; ++pass) {
-    words[bt.counter(pass)] = reg_groups;
-    std::fill_n(words + bt.counter(pass) + 1, n, 0);
+    words[bt.counter(pass)] = words[bt.counter(pass) + 1] = reg_groups;
+    std::fill_n(words + bt.counter(pass) + 2, n, (int)kLinkNone);
   }
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(g->d_table, g->h_table.data(), g->h_table.size(), cudaMemcpyHostToDevice, st);

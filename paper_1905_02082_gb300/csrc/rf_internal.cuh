@@ -501,9 +501,6 @@ __device__ __forceinline__ void st_relaxed_gpu_b128(ulonglong2* p, unsigned a, u
                : "memory");
 }
 
-__device__ __forceinline__ void st_relaxed_gpu_u32(unsigned* p, unsigned v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ void red_relaxed_gpu_add(unsigned* p, unsigned v) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -551,14 +548,15 @@ void prof_record(rf_volume* vol, int ev, cudaStream_t st);
 rf_status run_mesh(rf_volume* vol, float* verts, uint8_t* colors, int64_t cap, int64_t* n, cudaStream_t st);
 RegDesc make_reg_desc(rf_volume* vol, const DevFrame& f, const double* T_init, const uint8_t* mask, double* T_out,
                       rf_track_info* info);
-// Queue of a batch's registrations (device memory; see k_register_batch).
+// Queue of a batch's registrations (device memory; see rf_queue.hpp).
 struct RegQueue {
-  const int* cta_group;  // [CTAs]
-  const int* first;      // [groups + 1]
-  const int* order;      // [length] streams, in the order they are taken
-  unsigned* next;        // [groups], zero at the start
-  unsigned* counter;     // the number of groups at the start
+  const int* cta_group;   // [CTAs]
+  const int* first;       // [groups + 1]
+  const int* order;       // [length] streams, in the order they are taken
   const int* length;
+  unsigned* counter;      // next position to take: the number of groups at the start
+  unsigned* groups_left;  // groups that no member has closed: the same number
+  unsigned* links;        // [length], zero at the start
 };
 rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const RegQueue& q, int total_ctas,
                                 cudaStream_t st);

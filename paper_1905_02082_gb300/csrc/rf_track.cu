@@ -33,6 +33,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "rf_queue.hpp"
 #include "rf_volume.hpp"
 
 namespace rf {
@@ -922,56 +923,48 @@ __global__ void __launch_bounds__(kRegThreads, 1) k_register(RegDesc d) {
   register_body<ST, 1>(d, blockIdx.x, gridDim.x);
 }
 
+// The queue's memory operations (rf_queue.hpp) on the device: relaxed, at GPU
+// scope (the words carry all that they tell).
+struct QueueMem {
+  const RegDesc* descs;
+  const int* order;
+  __device__ unsigned load(const unsigned* p) { return ld_relaxed_gpu(p); }
+  __device__ unsigned add(unsigned* p, unsigned v) { return atomicAdd(p, v); }
+  __device__ unsigned cas(unsigned* p, unsigned expected, unsigned v) { return atomicCAS(p, expected, v); }
+  __device__ void pause(long long spins) {
+    if (spins > 4096) __nanosleep(64);
+  }
+  __device__ void abandon(int at) { atomicOr(descs[order[at]].status, ST_BARRIER); }
+};
+
+__device__ __noinline__ int next_stream(const RegDesc* descs, const RegQueue& q, int at, bool leader, long long limit) {
+  QueueMem mem = {descs, q.order};
+  return leader ? queue_lead(mem, q.links, q.counter, q.groups_left, at, *q.length)
+                : queue_follow(mem, q.links, at, *q.length, limit);
+}
+
 // The registrations of a batch in one cooperative launch.  CTA b is member
 // b - first[g] of group g = cta_group[b] (-1: no work) of first[g + 1] -
 // first[g] CTAs; groups never wait on each other.  A group registers the
-// streams of the queue one after the other: its first is order[g], its leader
-// takes the next from the shared counter and tells the group's other CTAs
-// through next[g] (round in the upper half, queue position + 1 in the lower).
+// streams of the queue one after the other (rf_queue.hpp).
 // Streams need 12 to 23 evaluations and have up to 12 times the pixels of
 // others; with a fixed set of streams per launch a quarter of the SMs' time was
 // spent waiting for the launch's last stream.  The queue and its counters
 // are part of the table that each call uploads.
 template <int ST>
-__global__ void __launch_bounds__(kRegThreads, 1)
-    k_register_batch(const RegDesc* __restrict__ descs, const int* __restrict__ cta_group, const int* __restrict__ first,
-                     const int* __restrict__ order, unsigned* next, unsigned* counter, const int* __restrict__ length) {
+__global__ void __launch_bounds__(kRegThreads, 1) k_register_batch(const RegDesc* __restrict__ descs,
+                                                                   const __grid_constant__ RegQueue q) {
   __shared__ RegDesc sd;
   __shared__ int s_at;
-  const int g = cta_group[blockIdx.x];
+  const int g = q.cta_group[blockIdx.x];
   if (g < 0) return;
-  const int lb = blockIdx.x - first[g], G = first[g + 1] - first[g], n = *length;
-  for (unsigned round = 0;; ++round) {
-    if (threadIdx.x == 0) {
-      int at = g;
-      if (round > 0) {
-        if (lb == 0) {
-          at = (int)atomicAdd(counter, 1u);
-          at = min(at, n);
-          st_relaxed_gpu_u32(next + g, (round << 16) | (unsigned)(at + 1));
-        } else {
-          // every member of the last registration has taken part in it, so it
-          // has read its round's word
-          unsigned w = 0u;
-          long long spins = 0;
-          for (;;) {
-            w = ld_relaxed_gpu(next + g);
-            if ((w >> 16) == round) break;
-            if (++spins > sd.spin_limit) {
-              atomicOr(sd.status, ST_BARRIER);
-              w = (unsigned)n + 1u;
-              break;
-            }
-            if (spins > 4096) __nanosleep(64);
-          }
-          at = (int)(w & 0xFFFFu) - 1;
-        }
-      }
-      s_at = at;
-    }
+  const int lb = blockIdx.x - q.first[g], G = q.first[g + 1] - q.first[g];
+  for (bool begun = false;; begun = true) {
+    if (threadIdx.x == 0)  // (there are no more groups than streams)
+      s_at = begun ? next_stream(descs, q, s_at, lb == 0, sd.spin_limit) : g;
     __syncthreads();
-    if (s_at >= n) return;
-    const RegDesc* from = descs + order[s_at];
+    if (s_at >= *q.length) return;
+    const RegDesc* from = descs + q.order[s_at];
     static_assert(sizeof(RegDesc) % 4 == 0, "copied in words");
     for (unsigned i = threadIdx.x; i < sizeof(RegDesc) / 4; i += kRegThreads)
       reinterpret_cast<unsigned*>(&sd)[i] = reinterpret_cast<const unsigned*>(from)[i];
@@ -1062,8 +1055,7 @@ rf_status launch_track(rf_volume* vol, const DevFrame& f, const double* T_init, 
 rf_status launch_register_batch(rf_volume* vol, const RegDesc* descs, const RegQueue& q, int total_ctas,
                                 cudaStream_t st) {
   RegQueue a = q;
-  void* args[] = {(void*)&descs, (void*)&a.cta_group, (void*)&a.first, (void*)&a.order,
-                  (void*)&a.next, (void*)&a.counter, (void*)&a.length};
+  void* args[] = {(void*)&descs, (void*)&a};
   const void* fn = vol->p.storage == RF_STORAGE_FP16 ? (const void*)k_register_batch<RF_STORAGE_FP16>
                                                      : (const void*)k_register_batch<RF_STORAGE_FP32>;
   return launch_coop(vol, fn, total_ctas, args, st);
