@@ -19,10 +19,12 @@
 // group is left, the rest of the queue.
 #pragma once
 
+#ifndef RF_HD
 #ifdef __CUDACC__
 #define RF_HD __host__ __device__ __forceinline__
 #else
 #define RF_HD inline
+#endif
 #endif
 
 namespace rf {

@@ -33,6 +33,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "rf_exchange.hpp"
 #include "rf_queue.hpp"
 #include "rf_volume.hpp"
 
@@ -543,6 +544,16 @@ __device__ __forceinline__ void write_record(const RegDesc& d, const Level& L, f
   d.rec[L.rec0 + i] = r;
 }
 
+// The counts' memory operations (rf_exchange.hpp) on the device.
+struct CountMem {
+  __device__ void red_relaxed(unsigned* p, unsigned v) { red_relaxed_gpu_add(p, v); }
+  __device__ unsigned add_acq_rel(unsigned* p, unsigned v) {
+    unsigned old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+  }
+};
+
 // Every CTA of a registration group calls this once, after its last use of
 // the exchange.  The last CTA to leave clears the arrival count and advances
 // the tag base past the
@@ -553,7 +564,10 @@ __device__ __forceinline__ void write_record(const RegDesc& d, const Level& L, f
 __device__ __forceinline__ void leave_registration(const RegDesc& d, int G, unsigned tag0) {
   __shared__ int s_last;
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(d.tags + 1, 1u) == (unsigned)G - 1u;
+  if (threadIdx.x == 0) {
+    CountMem mem;
+    s_last = last_to_leave(mem, d.tags + 1, (unsigned)G);
+  }
   __syncthreads();
   if (!s_last) return;
   const unsigned span = (unsigned)(d.c.iters[0] + d.c.iters[1] + d.c.iters[2] + 3);
@@ -598,6 +612,7 @@ __device__ __forceinline__ void register_body(const RegDesc& d, int lb, int G) {
   __shared__ RegShared S;
   __shared__ float red[2][kStepsPerBarrier][kRegWarps][32];  // per-warp sums of chunks, double-buffered
   constexpr int kRejectWarp = 12, kDecideWarp = 13;
+  CountMem count;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const DevFrame& f = d.f;
 
@@ -780,14 +795,14 @@ __device__ __forceinline__ void register_body(const RegDesc& d, int lb, int G) {
       if (lb < nchunks) {
         // arrival: one relaxed count per CTA (other warps' partial stores may
         // still be on their way: the readers check the tags)
-        if (threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
+        if (threadIdx.x == 0) arrive(count, d.tags + 2);
         // for the next evaluation, which samples the same pixels, during the
         // exchange: the first record
         int end;
         const int j = bounds(lb + G * slot, end);
         if (j < end) fetch(j);
       }
-      if (lb >= nchunks && threadIdx.x == 0) red_relaxed_gpu_add(d.tags + 2, 1u);
+      if (lb >= nchunks && threadIdx.x == 0) arrive(count, d.tags + 2);
       if (threadIdx.x == 0)
         S.arrived = await_count(d.tags + 2, (eval + 1u) * (unsigned)G + d.bar_extra - slack, d.spin_limit);
       // meanwhile: the next candidate should this one be rejected
