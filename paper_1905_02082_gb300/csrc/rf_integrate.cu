@@ -25,7 +25,11 @@
 //   k_nbr_fixup    neighbour tables of the blocks allocated
 // The four are short (3 to 25 us at 640x480), so each may start its CTAs while
 // its predecessor drains (programmatic dependent launch): it reads nothing
-// before griddepcontrol.wait has seen the predecessor complete.
+// before griddepcontrol.wait has seen the predecessor complete.  What the
+// predecessor writes is not constant over the kernel's life, so it is read by
+// ordinary loads, never through the read-only path (__ldg, or const with
+// __restrict__).  What an earlier kernel wrote may be: a kernel starts only
+// after every CTA of its predecessor has passed that wait.
 #include <cmath>
 
 #include "rf_volume.hpp"
@@ -44,7 +48,7 @@ __device__ __forceinline__ void start_successor() { asm volatile("griddepcontrol
 // Quantised pose (one entry per lane of warp 0: conversions run on the FP64
 // pipe, so they are spread over lanes), the per-frame constants of the voxel
 // loop and the reset of the per-frame counters.
-__device__ __forceinline__ void integ_prep(const double* __restrict__ T, IntegState* st, const int* __restrict__ n_blocks,
+__device__ __forceinline__ void integ_prep(const double* T, IntegState* st, const int* n_blocks,
                                            const DevParams& p) {
   const int a = threadIdx.x;
   if (a < 9) {
@@ -143,11 +147,10 @@ __device__ __forceinline__ void integ_aabb(const DevFrame& f, const DevParams& p
 // vec: rows of 8 pixels can be read and written with 16-byte accesses.
 constexpr int kTilesPerCta = 8;
 
-__global__ void __launch_bounds__(32 * kTilesPerCta) k_frustum(DevFrame f, DevParams p, const uint8_t* __restrict__ mask,
+__global__ void __launch_bounds__(32 * kTilesPerCta) k_frustum(DevFrame f, DevParams p, const uint8_t* mask,
                                                                int* __restrict__ tilemax, IntegState* st, int tiles_x,
                                                                int ntiles, uint16_t* __restrict__ dm,
-                                                               const double* __restrict__ T,
-                                                               const int* __restrict__ n_blocks, int vec) {
+                                                               const double* T, const int* n_blocks, int vec) {
   wait_for_predecessor();
   start_successor();
   if (gated_off(f.gate, kModeFirst)) return;
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(32 * kTilesPerCta) k_frustum(DevFrame f, DevPa
 
 // Conservative test: may keep blocks without updated voxels, never drops one.
 __device__ bool cull_keep(int bx, int by, int bz, const DevFrame& f, const DevParams& p, const IntegState& st,
-                          const int* __restrict__ tilemax, int tiles_x, int tiles_y, int max_um) {
+                          const int* tilemax, int tiles_x, int tiles_y, int max_um) {
   float zmin = 3.0e38f, zmax = -3.0e38f;
   float pcx[8], pcy[8], pcz[8];
 #pragma unroll
@@ -263,7 +266,7 @@ __device__ bool cull_keep(int bx, int by, int bz, const DevFrame& f, const DevPa
         int q[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k)
-          q[k] = __ldg(tilemax + min(ty + (k >> 2), ty1) * tiles_x + min(tx + (k & 3), tx1));
+          q[k] = tilemax[min(ty + (k >> 2), ty1) * tiles_x + min(tx + (k & 3), tx1)];
 #pragma unroll
         for (int k = 0; k < 16; ++k) m = max(m, q[k]);
       }
@@ -274,7 +277,7 @@ __device__ bool cull_keep(int bx, int by, int bz, const DevFrame& f, const DevPa
   return (float)m * 1e-6f + p.tau + eps >= zmin;
 }
 
-__global__ void __launch_bounds__(256) k_cull(DevFrame f, DevParams p, IntegState* st, const int* __restrict__ tilemax,
+__global__ void __launch_bounds__(256) k_cull(DevFrame f, DevParams p, IntegState* st, const int* tilemax,
                                               int tiles_x, int tiles_y, int4* __restrict__ cand, long long max_cand,
                                               unsigned* status) {
   wait_for_predecessor();
@@ -755,7 +758,7 @@ __device__ __forceinline__ void integ_flush(IntegState* st, unsigned updated, un
 template <int ST>
 __global__ void __launch_bounds__(kIntegThreads, 8) k_integrate(DevVol v, DevFrame f, DevParams p,
                                                              const uint16_t* __restrict__ dm, IntegState* st,
-                                                             const int4* __restrict__ cand, long long max_cand) {
+                                                             const int4* cand, long long max_cand) {
   __shared__ IntegShared sh;
   __shared__ unsigned short s_aq[kIntegWarps][kBV];  // voxels queued for the exact path
   __shared__ LaneConsts s_lc[kIntegThreads];
@@ -804,10 +807,10 @@ __device__ __forceinline__ void fixup_entry(const DevVol& v, int b, int k) {
   if (k == 0) {
     flat[8 * (size_t)b] = b;
   } else if (k < 8) {
-    flat[8 * (size_t)b + k] = hash_find(v, c.x + (k & 1), c.y + ((k >> 1) & 1), c.z + ((k >> 2) & 1));
+    flat[8 * (size_t)b + k] = hash_find<false>(v, c.x + (k & 1), c.y + ((k >> 1) & 1), c.z + ((k >> 2) & 1));
   } else {
     const int o = k - 7;
-    const int n = hash_find(v, c.x - (o & 1), c.y - ((o >> 1) & 1), c.z - ((o >> 2) & 1));
+    const int n = hash_find<false>(v, c.x - (o & 1), c.y - ((o >> 1) & 1), c.z - ((o >> 2) & 1));
     if (n >= 0) flat[8 * (size_t)n + o] = b;
   }
 }

@@ -204,14 +204,17 @@ __device__ __forceinline__ unsigned long long bucket_of(unsigned long long key, 
 }
 
 // Read-only lookup for kernels that do not insert (tracking, mask, mesh).
+// kConstant: the table does not change while the calling kernel lives, so the
+// read-only path may be used.
+template <bool kConstant = true>
 __device__ __forceinline__ int hash_find(const DevVol& v, int bx, int by, int bz) {
   if (!coord_ok(bx, by, bz)) return -1;
   const unsigned long long key = pack_key(bx, by, bz);
   const unsigned long long b = bucket_of(key, v.bucket_mask);
   for (int p = 0; p < kMaxProbe; ++p) {
     const ulonglong2* bp = reinterpret_cast<const ulonglong2*>(v.hash + ((b + p) & v.bucket_mask) * kSlots);
-    const ulonglong2 e01 = __ldg(bp);
-    const ulonglong2 e23 = __ldg(bp + 1);
+    const ulonglong2 e01 = kConstant ? __ldg(bp) : bp[0];
+    const ulonglong2 e23 = kConstant ? __ldg(bp + 1) : bp[1];
     const unsigned long long e[4] = {e01.x, e01.y, e23.x, e23.y};
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
