@@ -13,6 +13,7 @@
 #include "rf_cta_map.hpp"
 #include "rf_half.hpp"
 #include "rf_queue.hpp"
+#include "rf_reach.hpp"
 #include "rf_volume.hpp"
 
 namespace rf {
@@ -515,16 +516,53 @@ unsigned copy_ctas(const rf_volume* vol, size_t bytes) {
   return (unsigned)std::max<size_t>(1, std::min<size_t>((bytes / 16 + 255) / 256, 2 * (size_t)vol->sm_count));
 }
 
-// Whether kernels may read the memory at p: the device's own, or page-locked
-// host memory (which is what rf_frame documents; a pageable pointer goes
-// through the copy engine, as it did).
-bool kernel_readable(const void* p) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// Whether the volume's kernels may use the caller's buffer (rf_reach.hpp).
+bool kernel_reachable(const rf_volume* vol, const void* p, size_t bytes) {
+  return reachable(p, bytes, vol->device, [](cudaPointerAttributes* at, const void* q) {
+    const cudaError_t e = cudaPointerGetAttributes(at, q);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+  });
+}
+
+// A frame and its pose into the volume: one launch, or copies where a kernel
+// may not read some of them.
+rf_status frame_in(rf_volume* vol, const rf_frame* frame, const double* T, size_t npix, cudaStream_t st) {
+  if (kernel_reachable(vol, frame->depth, npix * 2) && kernel_reachable(vol, frame->rgb, npix * 3) &&
+      kernel_reachable(vol, T, 16 * sizeof(double))) {
+    const FrameIn in = {frame->depth, frame->rgb, T, vol->d_depth, vol->d_rgb, vol->d_T, npix};
+    k_frame_in<<<copy_ctas(vol, npix * 3), 256, 0, st>>>(in);
+    return check_cuda(vol, cudaGetLastError(), "frame staging");
   }
-  return at.type != cudaMemoryTypeUnregistered && at.devicePointer == p;
+  rf_status s = check_cuda(vol, cudaMemcpyAsync(vol->d_depth, frame->depth, npix * 2, cudaMemcpyDefault, st),
+                           "depth staging");
+  if (!s) s = check_cuda(vol, cudaMemcpyAsync(vol->d_rgb, frame->rgb, npix * 3, cudaMemcpyDefault, st), "rgb staging");
+  if (!s)
+    s = check_cuda(vol, cudaMemcpyAsync(vol->d_T, T, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st),
+                   "pose staging");
+  return s;
+}
+
+// A frame's results to the caller (mask and info may be NULL; a first frame's
+// info is zeros), likewise.
+rf_status frame_out(rf_volume* vol, bool first, double* T, uint8_t* mask, rf_track_info* info, size_t npix,
+                    cudaStream_t st) {
+  if (kernel_reachable(vol, T, 16 * sizeof(double)) && (!mask || kernel_reachable(vol, mask, npix)) &&
+      (!info || kernel_reachable(vol, info, sizeof(rf_track_info)))) {
+    const FrameOut out = {vol->d_T + 32, vol->d_mask, first ? nullptr : vol->d_info, T, mask, info, npix};
+    k_frame_out<<<copy_ctas(vol, mask ? npix : 0), 256, 0, st>>>(out);
+    return check_cuda(vol, cudaGetLastError(), "frame results");
+  }
+  rf_status s = check_cuda(vol, cudaMemcpyAsync(T, vol->d_T + 32, 16 * sizeof(double), cudaMemcpyDeviceToDevice, st),
+                           "pose out");
+  if (!s && mask)
+    s = check_cuda(vol, cudaMemcpyAsync(mask, vol->d_mask, npix, cudaMemcpyDeviceToDevice, st), "mask out");
+  if (!s && info)
+    s = check_cuda(vol,
+                   first ? cudaMemsetAsync(info, 0, sizeof(rf_track_info), st)
+                         : cudaMemcpyAsync(info, vol->d_info, sizeof(rf_track_info), cudaMemcpyDeviceToDevice, st),
+                   "info out");
+  return s;
 }
 
 rf_status batch_error(rf_batch* b, rf_status s, const std::string& msg) {
@@ -883,20 +921,9 @@ rf_status rf_process_frame(rf_volume* vol, const rf_frame* frame, const double* 
   cudaGraphExec_t exec = nullptr;
   rf_status s = vol->use_graphs ? frame_graph(vol, frame, first, &exec) : RF_OK;
   if (s) return s;
-  FrameIn in = {frame->depth, frame->rgb, T_init_dev, vol->d_depth, vol->d_rgb, vol->d_T, npix};
-  if (!kernel_readable(frame->depth) || !kernel_readable(frame->rgb)) {
-    if ((s = check_cuda(vol, cudaMemcpyAsync(vol->d_depth, frame->depth, npix * 2, cudaMemcpyDefault, st),
-                        "depth staging")) ||
-        (s = check_cuda(vol, cudaMemcpyAsync(vol->d_rgb, frame->rgb, npix * 3, cudaMemcpyDefault, st), "rgb staging")))
-      return s;
-    in.npix = 0;
-  }
-  k_frame_in<<<copy_ctas(vol, in.npix * 3), 256, 0, st>>>(in);
-  if ((s = check_cuda(vol, cudaGetLastError(), "frame staging"))) return s;
-  if ((s = run_frame(vol, frame, first, exec, st))) return s;
-  const FrameOut out = {vol->d_T + 32, vol->d_mask, first ? nullptr : vol->d_info, T_out_dev, mask_dev, info_dev, npix};
-  k_frame_out<<<copy_ctas(vol, mask_dev ? npix : 0), 256, 0, st>>>(out);
-  if ((s = check_cuda(vol, cudaGetLastError(), "frame results"))) return s;
+  if ((s = frame_in(vol, frame, T_init_dev, npix, st)) || (s = run_frame(vol, frame, first, exec, st)) ||
+      (s = frame_out(vol, first, T_out_dev, mask_dev, info_dev, npix, st)))
+    return s;
   vol->frames++;
   vol->has_model = true;
   return RF_OK;
