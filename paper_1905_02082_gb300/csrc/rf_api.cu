@@ -516,9 +516,9 @@ unsigned copy_ctas(const rf_volume* vol, size_t bytes) {
   return (unsigned)std::max<size_t>(1, std::min<size_t>((bytes / 16 + 255) / 256, 2 * (size_t)vol->sm_count));
 }
 
-// Whether the volume's kernels may use the caller's buffer (rf_reach.hpp).
-bool kernel_reachable(const rf_volume* vol, const void* p, size_t bytes) {
-  return reachable(p, bytes, vol->device, [](cudaPointerAttributes* at, const void* q) {
+// Whether the volume's staging kernels take the caller's buffer (rf_reach.hpp).
+bool by_kernel(const rf_volume* vol, const void* p, size_t bytes, size_t align) {
+  return staged_by_kernel(p, bytes, align, vol->device, [](cudaPointerAttributes* at, const void* q) {
     const cudaError_t e = cudaPointerGetAttributes(at, q);
     if (e != cudaSuccess) cudaGetLastError();
     return e;
@@ -526,10 +526,10 @@ bool kernel_reachable(const rf_volume* vol, const void* p, size_t bytes) {
 }
 
 // A frame and its pose into the volume: one launch, or copies where a kernel
-// may not read some of them.
+// may not read some of them or would be slow.
 rf_status frame_in(rf_volume* vol, const rf_frame* frame, const double* T, size_t npix, cudaStream_t st) {
-  if (kernel_reachable(vol, frame->depth, npix * 2) && kernel_reachable(vol, frame->rgb, npix * 3) &&
-      kernel_reachable(vol, T, 16 * sizeof(double))) {
+  if (by_kernel(vol, frame->depth, npix * 2, kImageAlign) && by_kernel(vol, frame->rgb, npix * 3, kImageAlign) &&
+      by_kernel(vol, T, 16 * sizeof(double), kWordAlign)) {
     const FrameIn in = {frame->depth, frame->rgb, T, vol->d_depth, vol->d_rgb, vol->d_T, npix};
     k_frame_in<<<copy_ctas(vol, npix * 3), 256, 0, st>>>(in);
     return check_cuda(vol, cudaGetLastError(), "frame staging");
@@ -547,8 +547,8 @@ rf_status frame_in(rf_volume* vol, const rf_frame* frame, const double* T, size_
 // info is zeros), likewise.
 rf_status frame_out(rf_volume* vol, bool first, double* T, uint8_t* mask, rf_track_info* info, size_t npix,
                     cudaStream_t st) {
-  if (kernel_reachable(vol, T, 16 * sizeof(double)) && (!mask || kernel_reachable(vol, mask, npix)) &&
-      (!info || kernel_reachable(vol, info, sizeof(rf_track_info)))) {
+  if (by_kernel(vol, T, 16 * sizeof(double), kWordAlign) && (!mask || by_kernel(vol, mask, npix, kImageAlign)) &&
+      (!info || by_kernel(vol, info, sizeof(rf_track_info), kWordAlign))) {
     const FrameOut out = {vol->d_T + 32, vol->d_mask, first ? nullptr : vol->d_info, T, mask, info, npix};
     k_frame_out<<<copy_ctas(vol, mask ? npix : 0), 256, 0, st>>>(out);
     return check_cuda(vol, cudaGetLastError(), "frame results");

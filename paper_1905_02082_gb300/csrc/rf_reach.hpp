@@ -4,6 +4,7 @@
 
 #include <cuda_runtime_api.h>
 #include <stddef.h>
+#include <stdint.h>
 
 namespace rf {
 
@@ -28,6 +29,18 @@ bool reachable(const void* p, size_t bytes, int device, Attributes&& attributes)
     }
     default: return false;
   }
+}
+
+// Images are copied 16 bytes at a time; byte by byte a kernel is slower than
+// the copy engine (an unaligned page-locked frame of 640x480: 23 us against
+// 13).  Poses and infos are accessed in 8 bytes, which a kernel may do only at
+// such an address.
+constexpr size_t kImageAlign = 16, kWordAlign = 8;
+
+// Whether the staging kernels take the buffer: reachable, at a multiple of `align`.
+template <class Attributes>
+bool staged_by_kernel(const void* p, size_t bytes, size_t align, int device, Attributes&& attributes) {
+  return reinterpret_cast<uintptr_t>(p) % align == 0 && reachable(p, bytes, device, attributes);
 }
 
 }  // namespace rf

@@ -32,7 +32,10 @@ def _run(R, snap, place):  # noqa: F811
         frame = R.rf_frame(cam.height, cam.width, cam.fx, cam.fy, cam.cx, cam.cy, depth.data_ptr(), colour.data_ptr())
         R.rf_process_frame(room.h, frame, pose, out, mask, info, None)
         room.sync()
-        got += [t.cpu().numpy().copy() for t in (out, mask, info)]
+        got += [t.cpu().numpy().copy() for t in (out, mask)]
+        i = R.rf_track_info.from_buffer_copy(info.cpu().numpy().tobytes())  # (field by field: it has padding)
+        got.append(np.hstack([np.ravel(np.ctypeslib.as_array(x) if hasattr(x, "__len__") else x).astype(np.float64)
+                              for x in (getattr(i, name) for name, _ in i._fields_)]))
     room.close()
     return got
 
@@ -57,3 +60,24 @@ def test_frame_and_results_in_other_memory(R, place):  # noqa: F811
     for a, b in zip(_run(R, snap, _device), _run(R, snap, place)):
         assert a.any()
         np.testing.assert_array_equal(a, b)
+
+
+def _offset(nbytes, pin=False):
+    def place(t):
+        raw = t.contiguous().view(torch.uint8).reshape(-1)
+        room = torch.zeros(raw.numel() + 16, dtype=torch.uint8)
+        room = room.pin_memory() if pin else room.cuda()
+        room[nbytes:nbytes + raw.numel()] = raw
+        return room[nbytes:nbytes + raw.numel()]
+    return place
+
+
+@pytest.mark.parametrize("nbytes,pin", [(2, False), (4, False), (8, False), (2, True)])
+def test_unaligned_frame_and_results(R, nbytes, pin):  # noqa: F811
+    """Views into larger buffers, as the frames of a stack whose frame size is
+    not a multiple of 16 bytes, at offsets that the images' element size allows."""
+    room = _room_volume(R)
+    snap = room.export()
+    room.close()
+    for a, b in zip(_run(R, snap, _device), _run(R, snap, _offset(nbytes, pin))):
+        np.testing.assert_array_equal(a.reshape(-1).view(np.uint8), b.reshape(-1).view(np.uint8))

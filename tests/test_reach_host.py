@@ -60,3 +60,33 @@ def test_buffers_that_kernels_may_use(driver):
     text = "".join("%d %d %d\n" % c for c, _ in CASES)
     out = subprocess.run([driver], input=text, capture_output=True, text=True, check=True).stdout
     assert [int(x) for x in out.split()] == [want for _, want in CASES]
+
+
+ALIGNED = r"""
+#include <cstdio>
+#include "rf_reach.hpp"
+int main() {
+  auto attributes = [](cudaPointerAttributes* at, const void* p) {
+    *at = cudaPointerAttributes{};
+    at->type = cudaMemoryTypeDevice;
+    return cudaSuccess;
+  };
+  for (unsigned long long p = 1 << 20; p < (1 << 20) + 32; ++p) {
+    const void* q = (const void*)(uintptr_t)p;
+    std::printf("%d %d\n", (int)rf::staged_by_kernel(q, 64, rf::kImageAlign, 0, attributes),
+                (int)rf::staged_by_kernel(q, 64, rf::kWordAlign, 0, attributes));
+  }
+  return 0;
+}
+"""
+
+
+def test_unaligned_buffers_go_to_the_copy_engine(tmp_path):
+    """The kernels copy images in 16-byte accesses, poses and infos in 8-byte ones."""
+    from paper_1905_02082_gb300.build import nvcc
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+    (tmp_path / "aligned.cpp").write_text(ALIGNED)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", CSRC, "-I", include, str(tmp_path / "aligned.cpp"), "-o",
+                    str(tmp_path / "aligned")], check=True)
+    out = subprocess.run([str(tmp_path / "aligned")], capture_output=True, text=True, check=True).stdout.split()
+    assert [int(x) for x in out] == [v for p in range(32) for v in (int(p % 16 == 0), int(p % 8 == 0))]
