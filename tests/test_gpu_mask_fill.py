@@ -127,3 +127,40 @@ def test_batch_masks_with_fewer_ctas_than_regions(R, oracle_mod):
     batch.close()
     for v in vols:
         v.close()
+
+
+def test_batch_masks_with_far_fewer_ctas_than_regions(R, oracle_mod):
+    """Enough 640x480 streams in one flood-fill launch that each has fewer CTAs
+    than regions whatever the kernel's occupancy (512 threads: at most 4 CTAs
+    per SM); the masks equal the oracle's at the streams' own poses."""
+    cam, regions = _camera(640, 480), 5 * 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 4 * sms // regions + 1
+    assert n <= sms and 4 * sms // n < regions
+    orc, snap = _model(oracle_mod, cam)
+    _, rgb = fronto_plane_frame(cam, PLANE)
+    depths = [_maze(640, 480, p) for p in ("rows", "columns", "random")]
+    depths[0][200:280] = PLANE - 50  # (open bands: the full corridors would take over a thousand sweeps)
+    depths[1][:, 280:360] = PLANE - 50
+    vols = [_volume(R, cam, snap) for _ in range(n)]
+    cfg = vols[0].launch_config()
+    cfg.batch_group = 0
+    vols[0].set_launch_config(cfg)
+    frames = [_device_frame(R, v, depths[k % 3], rgb, cam) for k, v in enumerate(vols)]
+    T0 = torch.eye(4, dtype=torch.float64, device="cuda")
+    # the pose of a stream's mask: its first registration, as the batch's bit for bit
+    poses = [vols[k].track(frames[k], T0)[0].cpu().numpy() for k in range(3)]
+    outs = [torch.empty(4, 4, dtype=torch.float64, device="cuda") for _ in vols]
+    masks = [torch.empty(480, 640, dtype=torch.uint8, device="cuda") for _ in vols]
+    batch = R.Batch(vols)
+    batch.process(frames, [T0] * n, outs, masks)
+    for v in vols:
+        v.sync()
+    want = [orc.compute_mask(oracle_mod.FrameData(d, rgb, cam.fx, cam.fy, cam.cx, cam.cy), T)
+            for d, T in zip(depths, poses)]
+    assert all(w.any() for w in want) and max(int(w.sum()) for w in want) > 1000
+    for k in range(n):
+        np.testing.assert_array_equal(masks[k].cpu().numpy(), want[k % 3])
+    batch.close()
+    for v in vols:
+        v.close()
