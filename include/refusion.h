@@ -142,7 +142,10 @@ rf_status rf_default_params(rf_params* p);
  * blocks allocated on demand, indexed by a spatial hash).  n_buckets must be
  * a power of two (4 slots per bucket); max_blocks <= 4,194,302.  max_width and
  * max_height bound the frames this volume accepts (per-frame scratch is sized
- * from them).  All device memory is allocated here.  On error *out is NULL. */
+ * from them; the largest part is 16 bytes per pixel that a registration samples,
+ * over its three levels: 174 MB at 3840 x 2160 and the default strides, instead
+ * of the candidate list where that is larger).  All device memory is
+ * allocated here.  On error *out is NULL. */
 rf_status rf_create_volume(const rf_params* p, int64_t n_buckets, int64_t max_blocks, int max_width,
                            int max_height, rf_volume** out);
 
@@ -174,7 +177,8 @@ rf_status rf_track_frame(rf_volume* vol, const rf_frame* frame, const double* T_
  * flood fill of Alg. 1 (4-neighbours, |D(p)-D(n)| < theta D(p)), 3x3
  * dilation.  mask_dev: device uint8 height*width (caller-owned output).
  * Seeds are decided exactly: near the threshold the residual is re-evaluated
- * in FP64 in a fixed operation order.  Asynchronous. */
+ * in float pairs, and near it still in FP64 in a fixed operation order.
+ * Asynchronous. */
 rf_status rf_compute_mask(rf_volume* vol, const rf_frame* frame, const double* T_dev, uint8_t* mask_dev,
                           void* stream);
 
@@ -223,7 +227,8 @@ rf_status rf_integrate_frame(rf_volume* vol, const rf_frame* frame, const double
  * round(d_max * depth_scale): the clipping plane, so that such rays carve free
  * space up to it); non-zero pixels are copied.  depth_out: device uint16
  * height*width; it may be frame->depth itself (in-place fill).  Decisions are
- * exact: FP32 with an error bound, FP64 re-evaluation near it.  Asynchronous. */
+ * exact: FP32 with an error bound, near it float pairs, then FP64.  Frames of
+ * more than 4 max_candidates pixels return RF_ERR_CAPACITY.  Asynchronous. */
 rf_status rf_virtual_depth(rf_volume* vol, const rf_frame* frame, const double* T_dev, int far_raw,
                            uint16_t* depth_out, void* stream);
 

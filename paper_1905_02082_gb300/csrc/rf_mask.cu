@@ -81,7 +81,7 @@ __device__ __forceinline__ int seed_of(const DevParams& p, const float F[8], con
 
 // Seed decision of one valid pixel in FP32 with an error bound: 0 or 1, or
 // 2 when the lattice cell or the comparison lies within the bound (the pixel
-// is then decided in FP64).  Rf: the pose as floats (R row-major, then t).
+// is then decided in float pairs or FP64).  Rf: the pose as floats (R row-major, then t).
 template <int ST>
 __device__ __forceinline__ int seed_fp32(const DevVol& v, const DevFrame& f, const DevParams& p, const float* Rf, int u,
                                          int vv, unsigned raw, unsigned long long cached) {

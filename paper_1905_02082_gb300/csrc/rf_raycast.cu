@@ -302,7 +302,8 @@ rf_status launch_virtual_depth(rf_volume* vol, const DevFrame& f, const double* 
   const double znear_d = vol->p.z_near, delta_d = vol->p.voxel_size * 0.5;
   const long long npix = (long long)f.H * f.W;
   if (npix > 4 * vol->p.max_candidates)
-    return set_error(vol, RF_ERR_CAPACITY, "frame larger than the hole list (4 x max_candidates pixels)");
+    return set_error(vol, RF_ERR_CAPACITY, "virtual depth: frame larger than 4 x max_candidates pixels");
+  // (the buffer holds any frame of the volume; the limit is the documented one)
   // scratch: the hole list and the crossings in the candidate buffer, counters
   // in the mask words (the guard count reports the samples FP32 left open)
   int* list = reinterpret_cast<int*>(vol->d_cand);

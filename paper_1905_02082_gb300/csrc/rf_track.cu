@@ -358,7 +358,7 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
 }
 
 // a * na < b * nb, exactly, for finite floats a, b >= 0 and integers
-// 0 <= na, nb < 2^24 (each product is a 48-bit integer times a power of two).
+// 0 <= na, nb < 2^32 (each product is a 56-bit integer times a power of two).
 __device__ __forceinline__ bool prod_less(float a, unsigned na, float b, unsigned nb) {
   const unsigned ba = __float_as_uint(a), bb = __float_as_uint(b);
   const unsigned ea = (ba >> 23) & 255u, eb = (bb >> 23) & 255u;
@@ -882,7 +882,7 @@ __device__ __forceinline__ void register_body(const RegDesc& d, int lb, int G) {
       }
       if (warp == kDecideWarp && lane == 0) {
         const float En = sums[27];
-        const unsigned Nn = (unsigned)(sums[28] + 0.5f);  // below 2^24, as the comparison's factors must be
+        const unsigned Nn = (unsigned)(sums[28] + 0.5f);  // exact up to 2^24 samples, then rounded as a float
         const bool enough = (long long)Nn >= d.c.min_valid;
         const bool accept = first || (enough && prod_less(En, S.N, S.E, Nn));
         S.info.evals++;

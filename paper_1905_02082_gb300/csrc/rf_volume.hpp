@@ -60,7 +60,7 @@ struct rf_volume {
   double* d_T = nullptr;        // [3][16]: T_in, T_first, T_second
   rf_track_info* d_info = nullptr;
 
-  unsigned* d_guard = nullptr;  // FP64 re-evaluated seed count of the last mask (d_ff[0])
+  unsigned* d_guard = nullptr;  // seeds (ray samples) that FP32 left open in the last mask (virtual depth): d_ff[0]
   unsigned long long* d_pxcache = nullptr;  // per pixel: block key << 22 | pool of its last sample
 
   // profiling: events recorded around the stages of the whole-frame calls
