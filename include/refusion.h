@@ -239,7 +239,9 @@ rf_status rf_virtual_depth(rf_volume* vol, const rf_frame* frame, const double* 
  * T_init_dev (in), T_out_dev (out), mask_dev (out, nullable), info_dev (out,
  * nullable; info of the second registration).  The frame is copied into
  * volume-owned staging buffers first, so the caller may reuse its buffers once
- * the stream passes this call.  The device work is replayed from a CUDA graph
+ * the stream passes this call: by a kernel from this device's and from
+ * page-locked memory (images at 16-byte boundaries), else by copies, as from
+ * another device's or from pageable memory.  The device work is replayed from a CUDA graph
  * captured per (frame size, intrinsics, first-frame) combination.
  * Asynchronous. */
 rf_status rf_process_frame(rf_volume* vol, const rf_frame* frame, const double* T_init_dev, double* T_out_dev,
@@ -270,7 +272,8 @@ rf_status rf_process_frame_host(rf_volume* vol, int height, int width, const dou
  * shape (frame sizes and intrinsics) captures a graph and allocates its small
  * descriptor buffers on first use.
  * rf_batch_process: frames, T_init_dev, T_out_dev, mask_dev (nullable, and
- * entries nullable) are arrays of n, device pointers as in rf_process_frame.
+ * entries nullable) are arrays of n; the batch's kernels access them, so they
+ * lie in its own device's or in page-locked memory.
  * A stream whose frames[i].depth is NULL sits the call out: its volume is left
  * unchanged, T_out_dev[i] receives T_init_dev[i], its mask is not written (its
  * frame's size and intrinsics must still be the stream's).  A stream whose
